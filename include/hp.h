@@ -159,7 +159,7 @@ enum {
                           A local-Laplacian level (K = 8, f32 stages; level 0 from u16 RGB): the same
                           30-column strips (of the coarser level), tile_h coarse rows per run.  Other
                           groups ignore HP_IMPL_WAVE's request when they have no streaming kernel. */
-  HP_IMPL_LINES = 3     /* line-buffer stencil chain: a chain of an even number of 5x5 stencils (2..8)
+  HP_IMPL_LINES = 3,    /* line-buffer stencil chain: a chain of an even number of 5x5 stencils (2..8)
                           whose input, stages and output share one type (f32, f16 or bf16; 16-bit
                           chains of 4 or 8 stages) runs as one thread block per tile_w x tile_h output
                           tile (tile_w a multiple of 8, tile_w + 4 depth <= 256 columns, tile_h >=
@@ -167,6 +167,11 @@ enum {
                           own and passes its rows to the next stage through a shared-memory ring
                           (threads and serial_y do not apply).  Other groups, and chains outside these
                           limits, ignore the request and take their default kernel. */
+  HP_IMPL_RESIDENT = 4  /* register-resident stencil chain: a chain of 2..16 5x5 stencils whose input,
+                          stages and output share one type (f32, f16 or bf16); a thread keeps 8 columns
+                          x serial_y rows (5, 6, 8, 9, 11, 14, 17 or 20) of a 256-column tile in
+                          registers through every stage.  serial_y and threads 0: chosen for the image; tile_w and
+                          tile_h follow.  Other groups ignore the request and take their default kernel. */
 };
 
 typedef struct {
@@ -238,8 +243,10 @@ enum {
   HP_KERNEL_GRID_SLICE = 22,    /* bilateral grid slice: four pixels of a row per thread, trilinear */
   HP_KERNEL_GRID_BLUR = 23,     /* bilateral grid blur (range levels, x, y; binomial/16), streaming:
                                   one warp per 28 grid columns x 4 range levels, y taps in order */
-  HP_KERNEL_STENCIL_LINES = 24  /* fused chain of 5x5 stencils, line-buffered: every stage on threads of
+  HP_KERNEL_STENCIL_LINES = 24, /* fused chain of 5x5 stencils, line-buffered: every stage on threads of
                                   its own, rows passed through shared-memory rings (HP_IMPL_LINES) */
+  HP_KERNEL_STENCIL_RESIDENT = 25 /* fused chain of 5x5 stencils, the tile in registers from the first
+                                  stage to the last (HP_IMPL_RESIDENT) */
 };
 
 /* Create an empty pipeline with n_inputs inputs of the given dtypes and channel

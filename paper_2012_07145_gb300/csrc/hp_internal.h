@@ -281,6 +281,11 @@ bool chain_lines_ok(int depth, int tile_w, int tile_h, int dtype);
 int chain_lines_threads(int depth, int tile_w, int tile_h, int dtype);
 int chain_lines_smem_bytes(int depth, int tile_w, int tile_h, int dtype);
 int launch_chain_lines(const ChainArgs& a, void* stream);
+// register-resident stencil chain (up to kResidentMaxDepth stages of one storage type)
+constexpr int kResidentMaxDepth = 16;
+int resident_shape(ChainArgs& a, int w, int h, int planes);
+int resident_smem_bytes(int threads);
+int launch_chain_resident(const ChainArgs& a, void* stream);
 int launch_generic(const GPlan& g, int threads, int smem_bytes, void* stream);
 int launch_pointwise(const PointwiseArgs& a, void* stream);
 int launch_downsample(const ResampleArgs& a, void* stream);

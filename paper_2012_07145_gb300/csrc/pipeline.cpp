@@ -934,6 +934,39 @@ hp_status build_chain_lines(const hp_pipeline* p, const Plan& plan, GroupPlan& g
   return HP_OK;
 }
 
+// Whether a chain group can take the register-resident kernel: the input,
+// every stage and the output stored in one type (f32, f16 or bf16), at most
+// kResidentMaxDepth stages.
+bool chain_resident_group_ok(const hp_pipeline* p, const GroupPlan& gp) {
+  const int in_dt = stage_dtype_of_ref(p, p->stages[gp.members[0]].inputs[0]);
+  if (in_dt != HP_F32 && in_dt != HP_F16 && in_dt != HP_BF16) return false;
+  for (int m : gp.members)
+    if (p->stages[m].storage != in_dt) return false;
+  return (int)gp.members.size() <= kResidentMaxDepth;
+}
+
+// A chain on the register-resident kernel: tiles of 256 columns (halo
+// included); the rows per thread (serial_y) and threads are chosen for the
+// image unless the schedule gives them.
+hp_status build_chain_resident(const hp_pipeline* p, const Plan& plan, GroupPlan& gp) {
+  chain_common_args(p, gp, false);
+  ChainArgs& a = gp.chain;
+  Dom od = plan.dom[gp.output];
+  const int planes = p->stages[gp.output].channels;
+  if (resident_shape(a, od.w, od.h, planes))
+    return fail(HP_ERR_SCHEDULE, "the register-resident chain kernel has no tile of %d rows per thread and %d threads "
+                                 "for %d stages (0: chosen)", gp.seg, gp.threads, a.depth);
+  gp.tile_w = a.tile_w;
+  gp.tile_h = a.tile_h;
+  gp.threads = a.threads;
+  gp.seg = a.seg;
+  gp.smem = resident_smem_bytes(a.threads);
+  gp.grid_x = a.tiles_x;
+  gp.grid_y = a.tiles_y;
+  gp.grid_z = planes;
+  return HP_OK;
+}
+
 // A chain of 2 or 4 stencils on the streaming kernel: strips of
 // chain_rows_strip_w columns, tile_h rows per run, every stage in registers.
 hp_status build_chain_rows(const hp_pipeline* p, const Plan& plan, GroupPlan& gp) {
@@ -1245,7 +1278,12 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
         gp.tile_h = pick(p->tile_h, g, streaming ? 0 : 32);  // 0: the streaming kernels' adaptive run length
         gp.threads = pick(p->threads, g, 256);
         gp.seg = pick(p->serial_y, g, 8);
-        if (!single && impl == HP_IMPL_LINES && chain_lines_group_ok(p, gp)) {
+        if (!single && impl == HP_IMPL_RESIDENT && chain_resident_group_ok(p, gp)) {
+          gp.kernel = HP_KERNEL_STENCIL_RESIDENT;
+          gp.threads = pick(p->threads, g, 0);  // 0: chosen for the image
+          gp.seg = pick(p->serial_y, g, 0);
+          s = build_chain_resident(p, plan, gp);
+        } else if (!single && impl == HP_IMPL_LINES && chain_lines_group_ok(p, gp)) {
           gp.kernel = HP_KERNEL_STENCIL_LINES;
           s = build_chain_lines(p, plan, gp);
         } else if (single && streaming) {
@@ -1610,7 +1648,8 @@ hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, c
       case HP_KERNEL_STENCIL_CHAIN:
       case HP_KERNEL_UNSHARP:
       case HP_KERNEL_STENCIL_WAVE:
-      case HP_KERNEL_STENCIL_LINES: {
+      case HP_KERNEL_STENCIL_LINES:
+      case HP_KERNEL_STENCIL_RESIDENT: {
         ChainArgs a = gp.chain;
         int first = gp.members[0];
         a.in = ref_view(p, plan, p->stages[first].inputs[0], inputs, output);
@@ -1618,6 +1657,7 @@ hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, c
         a.err = p->d_err;
         e = gp.kernel == HP_KERNEL_STENCIL_WAVE    ? launch_chain_rows(a, a.cols, a.tile_h, gp.grid_x, gp.smem, stream)
             : gp.kernel == HP_KERNEL_STENCIL_LINES ? launch_chain_lines(a, stream)
+            : gp.kernel == HP_KERNEL_STENCIL_RESIDENT ? launch_chain_resident(a, stream)
                                                    : launch_chain(a, gp.smem, stream);
         break;
       }
@@ -1922,7 +1962,7 @@ hp_status hp_schedule_set(hp_pipeline* p, const hp_schedule* s) {
   if ((st = per_group(s->tile_w, tmp.tile_w, 1, 4096, "tile_w")) || (st = per_group(s->tile_h, tmp.tile_h, 1, 4096, "tile_h")) ||
       (st = per_group(s->threads, tmp.threads, 32, 1024, "threads")) ||
       (st = per_group(s->serial_y, tmp.serial_y, 1, 256, "serial_y")) ||
-      (st = per_group(s->impl, tmp.impl, 0, 3, "impl")))
+      (st = per_group(s->impl, tmp.impl, 0, HP_IMPL_RESIDENT, "impl")))
     return st;
   std::vector<GroupShape> shapes;
   if ((st = group_shapes(&tmp, shapes))) return st;

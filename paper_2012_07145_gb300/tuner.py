@@ -10,7 +10,8 @@ sequence, not a compile.  The candidate spaces follow Sec. 4.1-4.3:
   - the kernel of a fused group: tiled (tile width 32/64/128, tile height a
     power of two, threads per block, serial rows per thread -- 4, 8, 16), or
     streaming (one warp per column strip, 4 or 8 columns per lane, rows per
-    run, threads per block), or the generic interpreter,
+    run, threads per block), or register-resident (tile shape chosen by the
+    library), or the generic interpreter,
   - for the local Laplacian, per pyramid level: streaming or tiled kernels,
     rows per run and threads,
 
@@ -133,6 +134,14 @@ def chain_candidates(n_stages, W, H, quick=False, esize=4):
     return out
 
 
+def resident_candidates(n_stages):
+    """The register-resident chain kernel: stages per launch (its tile shape is
+    chosen for the image)."""
+    from . import hp
+    return [dict(depth=d, tile_w=0, tile_h=0, threads=0, serial_y=0, impl=hp.HP_IMPL_RESIDENT)
+            for d in (2, 4, 8, 16) if n_stages % d == 0]
+
+
 # ----------------------------------------------------------- applications --
 def apply_schedule(p, entry):
     """Applies an application schedule (the params of a Harris, unsharp or
@@ -195,7 +204,8 @@ def workload(pipeline, w, h, dtype):
         n = int(n)
         return dict(kind="chain", build=lambda: (pipelines.stencil_chain(n, pattern, storage=st), None),
                     inputs=lambda: [(synth.stencil_input(h, w, seed=0), st)], out=(1, h, w, st),
-                    candidates=lambda quick: chain_candidates(n, w, h, quick, 4 if st == hp.HP_F32 else 2),
+                    candidates=lambda quick: chain_candidates(n, w, h, quick, 4 if st == hp.HP_F32 else 2)
+                    + resident_candidates(n),
                     apply=lambda p, ids, c: pipelines.chain_schedule(p, **c))
     if pipeline in ("harris", "unsharp", "histeq"):
         if pipeline == "harris":
@@ -262,6 +272,24 @@ def time_candidate(p, bi, bo, stream, flush, reps=15, probe=False):
     return (ms, attrs) if probe else ms
 
 
+def burst_ms(wl, p, ids, c, bi, bo, stream, n=200):
+    """Mean ms of back-to-back graph replays of candidate c (best of 3 bursts)."""
+    import torch
+    wl["apply"](p, ids, c)
+    best = float("inf")
+    for _ in range(3):
+        for _ in range(3):
+            p.realize(bi, bo, stream.cuda_stream)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record(stream)
+        for _ in range(n):
+            p.realize(bi, bo, stream.cuda_stream)
+        b.record(stream)
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) / n)
+    return best
+
+
 def tune(pipeline, w, h, dtype, quick=False, log=print):
     """Times every candidate of the workload (pruning on hardware limits and
     spills), checks each bit for bit against the stage-per-kernel result, and
@@ -315,6 +343,11 @@ def tune(pipeline, w, h, dtype, quick=False, log=print):
         log(f"{ms:.4f} ms {c}")
     results.sort(key=lambda r: r[0])
     best = results[0]
+    # event times come in steps of about 2 us: candidates within one step of the
+    # best are told apart by bursts of replays
+    near = [r for r in results if r[0] <= best[0] + 0.0025][:24]
+    if best[0] < 0.05 and len(near) > 1:
+        best = min(near, key=lambda r: burst_ms(wl, p, ids, r[1], bi, hp.buffer_from_tensor(y, odt), stream))
     return dict(workload=dict(pipeline=pipeline, w=w, h=h, dtype=dtype), kind=wl["kind"], params=best[1],
                 ms=best[0], plain_ms=plain_ms, registers=best[2], candidates=len(results),
                 pruned_spills=len(pruned), top5=[dict(ms=m, registers=r, **c) for m, c, r in results[:5]],
