@@ -1388,6 +1388,7 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
         a.st_mid = first.storage;
         a.st_out = last.storage;
         gp.ext_refs.assign(1, first.inputs[0]);
+        a.in.dtype = stage_dtype_of_ref(p, first.inputs[0]);
         gp.tile_w = max_rows_strip_w();
         gp.threads = pick(p->threads, g, 256);
         if (gp.threads % 32 != 0 || gp.threads < 32 || gp.threads > 256) {
@@ -1400,12 +1401,15 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
         const int strips = (od.w + gp.tile_w - 1) / gp.tile_w;
         gp.tile_h = pick(p->tile_h, g, 0);
         if (gp.tile_h == 0) {
-          a.in.dtype = stage_dtype_of_ref(p, first.inputs[0]);
-          gp.tile_h = default_run_rows(od.h, strips * planes,
-                                       (long long)max_rows_grid(a, 1 << 30, gp.threads) * (gp.threads / 32));
+          // one run per resident warp, not a few more (the last wave would
+          // hold only those); run and warm-up rows a whole number of boxes
+          const long long warps = (long long)max_rows_grid(a, 1 << 30, gp.threads) * (gp.threads / 32);
+          const long long runs = std::max(1LL, warps / std::max(1, strips * planes));
+          const int warm = a.shape == 1 ? 0 : 2 * a.radius;
+          const int rows = (int)std::max(8LL, (od.h + runs - 1) / runs);
+          gp.tile_h = (rows + warm + 3) / 4 * 4 - warm;
         }
         a.rows = gp.tile_h;
-        a.in.dtype = stage_dtype_of_ref(p, first.inputs[0]);
         gp.grid_x = max_rows_grid(a, strips * planes * ((od.h + a.rows - 1) / a.rows), gp.threads);
         gp.grid_y = 1;
         gp.smem = max_rows_smem_bytes(a, gp.threads);

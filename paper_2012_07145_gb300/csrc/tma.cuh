@@ -90,8 +90,9 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
 }
 
 // Host: encodes a 3-D (W, H, C) tiled tensor map with a (bw, bh, bz) box.
+// nan_fill: elements outside the image arrive as NaN (float types), else as 0.
 // Returns 0 on success.
 int encode_tmap_3d(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void* base, int w, int h, int c,
-                   long long row_stride, long long plane_stride, int bw, int bh, int bz = 1);
+                   long long row_stride, long long plane_stride, int bw, int bh, int bz = 1, bool nan_fill = false);
 
 }  // namespace hp

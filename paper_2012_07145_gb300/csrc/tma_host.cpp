@@ -31,7 +31,7 @@ EncodeTiledFn encoder() {
 }  // namespace
 
 int encode_tmap_3d(CUtensorMap* map, CUtensorMapDataType dt, int esize, const void* base, int w, int h, int c,
-                   long long row_stride, long long plane_stride, int bw, int bh, int bz) {
+                   long long row_stride, long long plane_stride, int bw, int bh, int bz, bool nan_fill) {
   EncodeTiledFn fn = encoder();
   if (!fn) return 1;
   if (((unsigned long long)base & 15) || row_stride % 16 || plane_stride % 16 || (bw * esize) % 16 || bw > 256 ||
@@ -43,7 +43,8 @@ int encode_tmap_3d(CUtensorMap* map, CUtensorMapDataType dt, int esize, const vo
   cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bz};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = fn(map, dt, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  nan_fill ? CU_TENSOR_MAP_FLOAT_OOB_FILL_NAN_REQUEST_ZERO_FMA : CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : 3;
 }
 
