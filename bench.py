@@ -88,7 +88,7 @@ def _chain_cfg(name, n, pattern, H, W, storage_name="f32"):
                 inputs=lambda seed: [(synth.stencil_input(H, W, seed=seed), st)], out=(1, H, W, st),
                 build=lambda: pipelines.stencil_chain(n, pattern, storage=st), fused=fused,
                 tuned_key=tkey, flops_px=flops_px, algorithmic=algorithmic, fp32_instr_px=10 * n,
-                bytes_px=2 * esize, bound="alu", kernel="k_chain", dtype=storage_name,
+                bytes_px=2 * esize, bound="alu", kernel="k_chain_resident", dtype=storage_name,
                 oracle_sample=oracle_sample, parity=parity, sample_rows=64,
                 lowp_error=lowp_error if storage_name != "f32" else None)
 

@@ -204,7 +204,8 @@ typedef struct {
 } hp_group_info;
 
 enum {
-  HP_KERNEL_STENCIL_CHAIN = 0, /* fused chain of 5x5 stencils (TMA tile + halo, register sweeps) */
+  HP_KERNEL_STENCIL_CHAIN = 0, /* fused chain of 5x5 stencils (TMA tile + halo, register sweeps; under
+                                  HP_IMPL_RESIDENT the tile in registers throughout) */
   HP_KERNEL_UNSHARP = 1,       /* 5x5 stencil + unsharp combine, fused */
   HP_KERNEL_HARRIS = 2,        /* whole Harris DAG in one kernel */
   HP_KERNEL_GENERIC = 3,       /* interpreter over any group of stencil/point-wise/pyramid stages */
@@ -243,10 +244,8 @@ enum {
   HP_KERNEL_GRID_SLICE = 22,    /* bilateral grid slice: four pixels of a row per thread, trilinear */
   HP_KERNEL_GRID_BLUR = 23,     /* bilateral grid blur (range levels, x, y; binomial/16), streaming:
                                   one warp per 28 grid columns x 4 range levels, y taps in order */
-  HP_KERNEL_STENCIL_LINES = 24, /* fused chain of 5x5 stencils, line-buffered: every stage on threads of
+  HP_KERNEL_STENCIL_LINES = 24  /* fused chain of 5x5 stencils, line-buffered: every stage on threads of
                                   its own, rows passed through shared-memory rings (HP_IMPL_LINES) */
-  HP_KERNEL_STENCIL_RESIDENT = 25 /* fused chain of 5x5 stencils, the tile in registers from the first
-                                  stage to the last (HP_IMPL_RESIDENT) */
 };
 
 /* Create an empty pipeline with n_inputs inputs of the given dtypes and channel

@@ -147,6 +147,7 @@ struct ChainArgs {
   int tile_w, tile_h, tiles_x, tiles_y;
   int threads, seg;
   int cols;                // streaming chain kernel: columns per lane (4 or 8)
+  int resident;            // the register-resident kernel (seg: rows per thread)
   int storage[kChainMax];
   float w[kChainMax][10];  // per stage: wx[5] then wy[5]
   int epilogue;            // 0: none; 1: unsharp out = in + amount*(in - chain(in))

@@ -423,6 +423,7 @@ int resident_shape(ChainArgs& a, int w, int h, int planes) {
     }
   }
   if (!found) return 1;
+  b.resident = 1;
   a = b;
   return 0;
 }

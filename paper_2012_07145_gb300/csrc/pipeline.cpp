@@ -1279,7 +1279,6 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
         gp.threads = pick(p->threads, g, 256);
         gp.seg = pick(p->serial_y, g, 8);
         if (!single && impl == HP_IMPL_RESIDENT && chain_resident_group_ok(p, gp)) {
-          gp.kernel = HP_KERNEL_STENCIL_RESIDENT;
           gp.threads = pick(p->threads, g, 0);  // 0: chosen for the image
           gp.seg = pick(p->serial_y, g, 0);
           s = build_chain_resident(p, plan, gp);
@@ -1652,8 +1651,7 @@ hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, c
       case HP_KERNEL_STENCIL_CHAIN:
       case HP_KERNEL_UNSHARP:
       case HP_KERNEL_STENCIL_WAVE:
-      case HP_KERNEL_STENCIL_LINES:
-      case HP_KERNEL_STENCIL_RESIDENT: {
+      case HP_KERNEL_STENCIL_LINES: {
         ChainArgs a = gp.chain;
         int first = gp.members[0];
         a.in = ref_view(p, plan, p->stages[first].inputs[0], inputs, output);
@@ -1661,7 +1659,7 @@ hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, c
         a.err = p->d_err;
         e = gp.kernel == HP_KERNEL_STENCIL_WAVE    ? launch_chain_rows(a, a.cols, a.tile_h, gp.grid_x, gp.smem, stream)
             : gp.kernel == HP_KERNEL_STENCIL_LINES ? launch_chain_lines(a, stream)
-            : gp.kernel == HP_KERNEL_STENCIL_RESIDENT ? launch_chain_resident(a, stream)
+            : a.resident ? launch_chain_resident(a, stream)
                                                    : launch_chain(a, gp.smem, stream);
         break;
       }

@@ -24,6 +24,11 @@ def resident(n, depth, rows, threads, dtype="f32"):
     return p
 
 
+def is_resident(info):
+    """The resident kernel's shared memory: two buffers of four 256-column f32 rows per warp."""
+    return info.kernel == hp.HP_KERNEL_STENCIL_CHAIN and info.smem_bytes == info.threads // 32 * 8192
+
+
 @pytest.mark.parametrize("h,w", SIZES + [(1536, 2560), (4097, 3001)])
 @pytest.mark.parametrize("depth", [2, 3, 4, 8])
 @pytest.mark.parametrize("rows,threads", [(20, 256), (11, 384), (5, 512), (9, 160)])
@@ -32,7 +37,7 @@ def test_tiles_cover_every_pixel_once(h, w, depth, rows, threads):
     pixels past the halo, the last one up to the image's end, and a tile holds
     2 depth pixels more on every side inside the image."""
     info = resident(depth, depth, rows, threads).group_info([(w, h)], 0)
-    assert info.kernel == hp.HP_KERNEL_STENCIL_RESIDENT and info.threads == threads
+    assert is_resident(info) and info.threads == threads
     full_y = rows * threads // 32
     hx, hy = (256 - info.tile_w) // 2, (full_y - info.tile_h) // 2
     if info.grid_x > 1 and info.grid_y > 1:
@@ -57,7 +62,7 @@ def test_shapes_out_of_range_are_refused_and_other_chains_keep_their_kernel():
     a = q.add_stage(hp.HP_STENCIL, [q.input(0)], 1, hp.HP_F16, rx=2, ry=2, wx=pipelines.BOX5, wy=pipelines.BOX5)
     q.set_output(q.add_stage(hp.HP_STENCIL, [a], 1, hp.HP_F16, rx=2, ry=2, wx=pipelines.BOX5, wy=pipelines.BOX5))
     q.schedule([0, 0], impl=[hp.HP_IMPL_RESIDENT])
-    assert q.group_info([(64, 48)], 0).kernel == hp.HP_KERNEL_STENCIL_CHAIN
+    assert not is_resident(q.group_info([(64, 48)], 0))
 
 
 def _base(n, h, w, dtype):
@@ -80,7 +85,7 @@ def test_bit_identical(h, w, dtype):
     for depth, rows, threads in [(16, 0, 0), (8, 0, 0), (4, 5, 128), (6, 6, 256), (8, 8, 512), (4, 9, 192),
                                  (8, 11, 384), (2, 14, 64), (4, 17, 256), (8, 20, 256), (16, 20, 256), (4, 5, 160)]:
         p = resident(n, depth, rows, threads, dtype)
-        assert p.group_info([(w, h)], 0).kernel == hp.HP_KERNEL_STENCIL_RESIDENT
+        assert is_resident(p.group_info([(w, h)], 0))
         n0 = hp.launch_count()
         y = run(p, [x], [ST[dtype]], (1, h, w), ST[dtype])
         assert hp.launch_count() - n0 == -(-n // depth)
