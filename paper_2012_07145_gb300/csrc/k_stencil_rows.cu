@@ -2,20 +2,21 @@
 // combine (out = in + amount (in - blur)), per channel plane.
 //
 // Each warp owns a strip of output columns, four per lane, of one plane and
-// walks down a run of rows.  Input rows arrive as TMA boxes (kBoxRows rows, 128
-// columns) through a ring of shared-memory slots private to the warp, so the
-// loads of later rows overlap the arithmetic on the current one and no barrier
-// wider than the warp is taken.  The x pass takes its two neighbours on each
-// side from the adjacent lanes (the outer lanes only feed them), the y pass
-// runs over a 5-row register window of x-pass results, and the unsharp
-// combine reads the input row from a matching 5-row window.  The stencil and
-// combine expressions are those of stage_math.cuh, so the result is
-// bit-identical to every other schedule of the pipeline.
+// walks down a run of rows, four at a time.  Input rows arrive as TMA boxes
+// (kBoxRows rows, 128 columns) through a ring of shared-memory slots private to
+// the warp, so the loads of later rows overlap the arithmetic on the current
+// ones and no barrier wider than the warp is taken.  A warp runs one unit (run of
+// rows) and every lane tests a box's barrier itself: a ring that ran on into the
+// warp's next unit, waited on by one lane, cost more in bookkeeping than the
+// arithmetic.  The x pass reads the two columns on either side from shared
+// memory, the y pass runs over the x-pass results of the last eight rows (two
+// blocks, alternating, so nothing is moved), and the unsharp combine keeps the
+// two input rows it is behind.  The stencil and combine expressions are those of
+// stage_math.cuh, so the result is bit-identical to every other schedule.
 //
 // Boundary condition (clamp to edge on the stencil's input): in strips that
-// touch the left or right image edge the input row's columns outside the image
-// take the edge column's value (shuffled from the lane that holds it); rows
-// outside take the nearest edge row's x-pass result (a copy inside the window).
+// touch the left or right image edge the two columns outside it are written into
+// the arrived box; rows outside take the nearest edge row's x-pass result.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -57,7 +58,7 @@ struct SRowsParams {
 };
 
 struct Unit {
-  int x0, oy, plane, n_in, nbox;  // x0: image column of lane 0's first column
+  int x0, oy, plane, nout, nbox;  // x0: image column of lane 0's first column
 };
 
 __device__ __forceinline__ Unit unit_geom(const SRowsParams& kp, const StripGeom& g, int u) {
@@ -68,65 +69,24 @@ __device__ __forceinline__ Unit unit_geom(const SRowsParams& kp, const StripGeom
   const int run = v / kp.strips, s = v - run * kp.strips;
   U.x0 = s * g.strip_w - 4 * g.halo_lanes;
   U.oy = run * kp.rows;
-  U.n_in = min(kp.rows, kp.a.out.h - U.oy) + 4;
-  U.nbox = (U.n_in + kBoxRows - 1) / kBoxRows;
+  U.nout = min(kp.rows, kp.a.out.h - U.oy);
+  U.nbox = (U.nout + 4 + kBoxRows - 1) / kBoxRows;
   return U;
 }
 
-// The warp's ring: box q (in issue order, which is the order of use) lives in
-// slot q % kRing and completes phase (q / kRing) & 1 of that slot's mbarrier.
-struct Ring {
-  unsigned char* slots;
-  uint64_t* bars;
-  unsigned issued, released;
-  int iu, ij;  // next box to issue: unit and box within it
-  Unit IU;     // geometry of unit iu
-};
-
-__device__ __forceinline__ void issue_one(const SRowsParams& kp, const StripGeom& g, Ring& R, int stride, int lane) {
-  if (R.iu >= kp.units) return;
-  if (lane == 0) {
-    const int s = R.issued % kRing;
-    mbar_arrive_expect_tx(R.bars + s, (unsigned)g.slot_bytes);
-    tma_load_3d(R.slots + s * g.slot_bytes, &kp.tmap, R.IU.x0, R.IU.oy - 2 + R.ij * kBoxRows, R.IU.plane,
-                R.bars + s);
-  }
-  ++R.issued;
-  if (++R.ij == R.IU.nbox) {
-    R.ij = 0;
-    R.iu += stride;
-    if (R.iu < kp.units) R.IU = unit_geom(kp, g, R.iu);
-  }
-}
-
-// Every lane's value at a column outside [0, W) becomes the value at the
-// nearest column inside, fetched from the lane that holds it.
-__device__ __forceinline__ void clamp_cols(float (&v)[4], int c0, int x0, int W) {
-  float o[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int c = c0 + k;
-    const int s = min(max(c, 0), W - 1);
-    const int off = s - x0;
-    const int sl = off >> 2, sk = off & 3;
-    const float t0 = __shfl_sync(kFull, v[0], sl), t1 = __shfl_sync(kFull, v[1], sl);
-    const float t2 = __shfl_sync(kFull, v[2], sl), t3 = __shfl_sync(kFull, v[3], sl);
-    const float t = sk == 0 ? t0 : sk == 1 ? t1 : sk == 2 ? t2 : t3;
-    o[k] = c == s ? v[k] : t;
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = o[k];
-}
-
-__device__ __forceinline__ void load4(const unsigned char* p, int dtype, float (&v)[4]) {
-  if (dtype == HP_F32) {
+// Four columns at p, and the two on either side.
+template <bool F32>
+__device__ __forceinline__ void load8(const unsigned char* p, int dtype, float (&v)[8]) {
+  if (F32 || dtype == HP_F32) {
+    const float2 l = *reinterpret_cast<const float2*>(p - 8);
     const float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    const float2 r = *reinterpret_cast<const float2*>(p + 16);
+    v[0] = l.x; v[1] = l.y; v[2] = q.x; v[3] = q.y; v[4] = q.z; v[5] = q.w; v[6] = r.x; v[7] = r.y;
   } else {
     const uint2 q = *reinterpret_cast<const uint2*>(p);
-    const unsigned u[2] = {q.x, q.y};
+    const unsigned u[4] = {*reinterpret_cast<const unsigned*>(p - 4), q.x, q.y, *reinterpret_cast<const unsigned*>(p + 8)};
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 4; ++i) {
       const unsigned short lo = (unsigned short)(u[i] & 0xffffu), hi = (unsigned short)(u[i] >> 16);
       if (dtype == HP_BF16) {
         v[2 * i] = __bfloat162float(__ushort_as_bfloat16(lo));
@@ -139,11 +99,6 @@ __device__ __forceinline__ void load4(const unsigned char* p, int dtype, float (
   }
 }
 
-// One run of rows of one strip of one plane.  Step t reads input row t
-// (image row oy - 2 + t) and, from t = 4 on, emits output row t - 4 of the
-// run.  Windows are indexed by row mod 5, so a loop unrolled five times keeps
-// them in fixed registers.  F32 = every storage type is f32 (no rounding, one
-// 128-bit store per lane and row).
 // The binomial [1,4,6,4,1]/16 taps (the unsharp blur, the same float values
 // the pipeline stores) as compile-time constants.
 __device__ __forceinline__ float tap5_binomial_const(float a, float b, float c, float d, float e) {
@@ -154,139 +109,169 @@ __device__ __forceinline__ float tap5_binomial_const(float a, float b, float c, 
   return __fmaf_rn(0.0625f, e, s);
 }
 
-// BIN: both passes take the binomial taps (checked bit for bit on the host),
-// compiled as constants: no registers for the taps, which lets the unsharp
-// kernel keep five CTAs of 128 threads per SM without spilling.
+// One run of rows of one strip of one plane.  Box i lives in slot i % kRing and
+// completes phase (i / kRing) & 1 of that slot's mbarrier; its rows are input
+// rows 4 i .. 4 i + 3 of the run (image rows oy - 2 + ...), and row t of the run
+// emits output row t - 4.  F32 = every storage type is f32 (no rounding, one
+// 128-bit store per lane and row).  BIN: both passes take the binomial taps
+// (checked bit for bit on the host), compiled as constants.
 template <bool F32, bool EPI, bool BIN>
 struct StripRun {
   const SRowsParams& kp;
   const StripGeom& g;
-  Ring& R;
-  const Unit U;
-  const int lane, stride, c0, esize;
-  const bool hb;             // the strip touches the left or right image edge
+  const Unit& U;
+  unsigned char* const slots;
+  uint64_t* const bars;
+  const int lane, c0, esize;
   const bool vedge;          // the run reads rows outside the image
   float wx[5], wy[5];
-  float hx[5][4];            // x-pass results
-  float raw[5][4];           // input values (for the unsharp combine)
-  bool st_full, st_part;     // the lane stores four columns / some of its columns
-  char* out_row;             // the next output row
-  unsigned q;                // box being read
-  int rr;                    // row within it
-  const unsigned char* slot;
+  bool vec, part, cut;       // the lane stores its four columns at once / one by one, up to the edge; any lane does
+  char* out_row;             // output row of the next input row
+  int s, phase;              // slot and phase of the next box
+  float behind[2][4];        // the last two input rows (unsharp)
 
-  __device__ __forceinline__ StripRun(const SRowsParams& kp_, const StripGeom& g_, Ring& R_, const Unit& U_,
-                                      int lane_, int stride_)
-      : kp(kp_), g(g_), R(R_), U(U_), lane(lane_), stride(stride_), c0(U_.x0 + 4 * lane_),
-        esize(kp_.a.in.dtype == HP_F32 ? 4 : 2), hb(U_.x0 < 0 || U_.x0 + 128 > kp_.a.in.w),
-        vedge(U_.oy < 2 || U_.oy + U_.n_in - 2 > kp_.a.in.h), q(R_.released),
-        rr(0), slot(nullptr) {
+  __device__ __forceinline__ StripRun(const SRowsParams& kp_, const StripGeom& g_, const Unit& U_, unsigned char* slots_,
+                                      uint64_t* bars_, int lane_)
+      : kp(kp_), g(g_), U(U_), slots(slots_), bars(bars_), lane(lane_), c0(U_.x0 + 4 * lane_),
+        esize(F32 || kp_.a.in.dtype == HP_F32 ? 4 : 2), vedge(U_.oy < 2 || U_.oy + U_.nout + 2 > kp_.a.in.h), s(0), phase(0) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       wx[k] = kp.a.w[0][k];
       wy[k] = kp.a.w[0][5 + k];
     }
-    const int W = kp.a.out.w;
-    const bool mine = lane >= g.halo_lanes && lane < 32 - g.halo_lanes;
-    st_full = mine && c0 + 3 < W && F32;
-    st_part = mine && c0 < W && !st_full;
-    out_row = (char*)kp.a.out.data + (long long)U.plane * kp.a.out.ps + (long long)U.oy * kp.a.out.rs;
+    const ImgView& ov = kp.a.out;
+    const bool mine = lane >= g.halo_lanes && lane < 32 - g.halo_lanes && c0 < ov.w;
+    const int osize = F32 ? 4 : dtype_size(ov.dtype);
+    vec = mine && c0 + 3 < ov.w && (osize == 4 ? ov.dtype == HP_F32 : osize == 2 && ov.dtype != HP_U16);
+    part = mine && !vec;
+    cut = __any_sync(kFull, part);
+    out_row = (char*)ov.data + (long long)U.plane * ov.ps + (long long)(U.oy - 4) * ov.rs + (long long)c0 * osize;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) behind[0][k] = behind[1][k] = 0.0f;
   }
 
-  __device__ __forceinline__ bool wait_box() {
-    int ok = 1;
-    if (lane == 0) ok = mbar_wait_poll(R.bars + q % kRing, (q / kRing) & 1u, 2000000000ull);
+  __device__ __forceinline__ void issue(int i, int slot) {
+    // the warp's accesses to this slot (its previous box) come before the copy
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive_expect_tx(bars + slot, (unsigned)g.slot_bytes);
+    tma_load_3d(slots + slot * g.slot_bytes, &kp.tmap, U.x0, U.oy - 2 + i * kBoxRows, U.plane, bars + slot);
+  }
+
+  // In a strip at the left or right edge: the two columns outside the image,
+  // where the box holds them, become the edge column (16 lanes, one value each).
+  __device__ __forceinline__ void fill_edges(unsigned char* box) {
+    const int W = kp.a.in.w;
+    const int row = lane & 3, k = (lane >> 2) & 1;
+    const int edge = (lane < 8 ? 0 : W - 1) - U.x0, to = lane < 8 ? edge - 1 - k : edge + 1 + k;
+    if (lane < 16 && edge >= 0 && edge < 128 && to >= 0 && to < 128) {
+      unsigned char* r = box + row * 128 * esize;
+      if (esize == 4) {
+        reinterpret_cast<float*>(r)[to] = reinterpret_cast<const float*>(r)[edge];
+      } else {
+        reinterpret_cast<unsigned short*>(r)[to] = reinterpret_cast<const unsigned short*>(r)[edge];
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before the slot's next copy
     __syncwarp();
-    ok = __shfl_sync(kFull, ok, 0);
-    slot = R.slots + (q % kRing) * g.slot_bytes + lane * 4 * esize;
-    return ok != 0;
   }
 
-  __device__ __forceinline__ void release_box() {
-    ++q;
-    __syncwarp();
-    R.released = q;
-    issue_one(kp, g, R, stride, lane);
+  __device__ __forceinline__ float tap_x(float a, float b, float c, float d, float e) const {
+    return BIN ? tap5_binomial_const(a, b, c, d, e) : tap5(wx, a, b, c, d, e);
+  }
+  __device__ __forceinline__ float tap_y(float a, float b, float c, float d, float e) const {
+    return BIN ? tap5_binomial_const(a, b, c, d, e) : tap5(wy, a, b, c, d, e);
   }
 
-  template <int M>
-  __device__ __forceinline__ bool step(int t) {
+  // Box i: A holds the x-pass results of the four rows before it, B receives its own.
+  __device__ __forceinline__ bool block(int i, float (&A)[4][4], float (&B)[4][4]) {
     const ChainArgs& a = kp.a;
-    const int r = U.oy - 2 + t;
-    if (rr == 0 && !wait_box()) return false;
-    float v[4];
-    load4(slot + rr * 128 * esize, F32 ? HP_F32 : a.in.dtype, v);
-    if (++rr == kBoxRows) {
-      rr = 0;
-      release_box();
-    }
-    if (hb) clamp_cols(v, c0, U.x0, a.in.w);
+    // every lane waits for the box itself (usually there: one test)
+    if (!__all_sync(kFull, mbar_try_wait(bars + s, phase) || mbar_wait_poll(bars + s, phase, 2000000000ull))) return false;
+    unsigned char* const box = slots + s * g.slot_bytes;
+    if (U.x0 < 0 || U.x0 + 128 > a.in.w) fill_edges(box);
+    const unsigned char* p = box + lane * 4 * esize;
+    float raw[4][4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) raw[M][k] = v[k];
-    // x pass: columns c0-2 .. c0+5
-    const float l2 = __shfl_up_sync(kFull, v[2], 1), l1 = __shfl_up_sync(kFull, v[3], 1);
-    const float r1 = __shfl_down_sync(kFull, v[0], 1), r2 = __shfl_down_sync(kFull, v[1], 1);
-    hx[M][0] = BIN ? tap5_binomial_const(l2, l1, v[0], v[1], v[2]) : tap5(wx, l2, l1, v[0], v[1], v[2]);
-    hx[M][1] = BIN ? tap5_binomial_const(l1, v[0], v[1], v[2], v[3]) : tap5(wx, l1, v[0], v[1], v[2], v[3]);
-    hx[M][2] = BIN ? tap5_binomial_const(v[0], v[1], v[2], v[3], r1) : tap5(wx, v[0], v[1], v[2], v[3], r1);
-    hx[M][3] = BIN ? tap5_binomial_const(v[1], v[2], v[3], r1, r2) : tap5(wx, v[1], v[2], v[3], r1, r2);
-    if (vedge && (r < 1 || r >= a.in.h)) {
-      if (r == 0) {  // rows -2 and -1 are row 0
+    for (int j = 0; j < 4; ++j) {
+      float v[8];
+      load8<F32>(p + j * 128 * esize, a.in.dtype, v);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { hx[(M + 3) % 5][k] = hx[M][k]; hx[(M + 4) % 5][k] = hx[M][k]; }
+      for (int k = 0; k < 4; ++k) {
+        raw[j][k] = v[k + 2];
+        B[j][k] = tap_x(v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4]);
       }
-      if (r >= a.in.h) {  // rows H and H + 1 are row H - 1
+      if (vedge) {
+        const int r = U.oy - 2 + 4 * i + j;
+        if (r == 0) {  // rows -2 and -1 are row 0 (rows 2 and up of the run: j >= 2)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) hx[M][k] = hx[(M + 4) % 5][k];
+          for (int k = 0; k < 4; ++k) { B[(j + 3) & 3][k] = B[j][k]; B[(j + 2) & 3][k] = B[j][k]; }
+        }
+        if (r >= a.in.h) {  // rows H and H + 1 are row H - 1
+#pragma unroll
+          for (int k = 0; k < 4; ++k) B[j][k] = j ? B[(j + 3) & 3][k] : A[3][k];
+        }
       }
-    }
-    if (t >= 4) {
-      // y pass over rows t-4 .. t -> output row t - 4 of the run (input row t - 2)
-      constexpr int J0 = (M + 1) % 5, J1 = (M + 2) % 5, J2 = (M + 3) % 5, J3 = (M + 4) % 5;
+      const int t = 4 * i + j - 4;   // output row of the run
+      const bool in_run = (unsigned)t < (unsigned)U.nout;
       float o[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        float b = BIN ? tap5_binomial_const(hx[J0][k], hx[J1][k], hx[J2][k], hx[J3][k], hx[M][k])
-                      : tap5(wy, hx[J0][k], hx[J1][k], hx[J2][k], hx[J3][k], hx[M][k]);
+        const float r0 = j < 1 ? A[0][k] : j < 2 ? A[1][k] : j < 3 ? A[2][k] : A[3][k];
+        const float r1 = j < 1 ? A[1][k] : j < 2 ? A[2][k] : j < 3 ? A[3][k] : B[0][k];
+        const float r2 = j < 1 ? A[2][k] : j < 2 ? A[3][k] : j < 3 ? B[0][k] : B[1][k];
+        const float r3 = j < 1 ? A[3][k] : j < 2 ? B[0][k] : j < 3 ? B[1][k] : B[2][k];
+        float b = tap_y(r0, r1, r2, r3, B[j][k]);
         if (!F32) b = round_storage(a.storage[0], b);
         if (EPI) {
-          b = op_unsharp(raw[J2][k], b, a.amount);
+          b = op_unsharp(j < 2 ? behind[j & 1][k] : raw[j < 2 ? 0 : j - 2][k], b, a.amount);
           if (!F32) b = round_storage(a.out.dtype, b);
         }
         o[k] = b;
       }
-      char* row = out_row;
-      out_row += a.out.rs;
-      if (st_full) {
-        *reinterpret_cast<float4*>(row + 4LL * c0) = make_float4(o[0], o[1], o[2], o[3]);
-      } else if (st_part) {
-        const int y = U.oy + t - 4;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (c0 + k < a.out.w) store_px(a.out, U.plane, c0 + k, y, o[k]);
+      if (vec && in_run) {
+        if (F32 || a.out.dtype == HP_F32) {
+          *reinterpret_cast<float4*>(out_row) = make_float4(o[0], o[1], o[2], o[3]);
+        } else if (a.out.dtype == HP_BF16) {
+          const __nv_bfloat162 q0 = __floats2bfloat162_rn(o[0], o[1]), q1 = __floats2bfloat162_rn(o[2], o[3]);
+          *reinterpret_cast<uint2*>(out_row) =
+              make_uint2(*reinterpret_cast<const unsigned*>(&q0), *reinterpret_cast<const unsigned*>(&q1));
+        } else {
+          const __half2 q0 = __floats2half2_rn(o[0], o[1]), q1 = __floats2half2_rn(o[2], o[3]);
+          *reinterpret_cast<uint2*>(out_row) =
+              make_uint2(*reinterpret_cast<const unsigned*>(&q0), *reinterpret_cast<const unsigned*>(&q1));
+        }
       }
+      if (cut) {
+        if (part && in_run) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (c0 + k < a.out.w) store_px(a.out, U.plane, c0 + k, U.oy + t, o[k]);
+        }
+      }
+      out_row += a.out.rs;
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { behind[0][k] = raw[2][k]; behind[1][k] = raw[3][k]; }
+    __syncwarp();   // every lane has read the box
+    if (lane == 0 && i + kRing < U.nbox) issue(i + kRing, s);
+    phase ^= s == kRing - 1;
+    s = s == kRing - 1 ? 0 : s + 1;
     return true;
   }
 
+  // False: a box never arrived.
   __device__ __forceinline__ bool run() {
-    const int n = U.n_in;
-    int t = 0;
-    while (true) {
-      if (!step<0>(t)) return false;
-      if (++t >= n) break;
-      if (!step<1>(t)) return false;
-      if (++t >= n) break;
-      if (!step<2>(t)) return false;
-      if (++t >= n) break;
-      if (!step<3>(t)) return false;
-      if (++t >= n) break;
-      if (!step<4>(t)) return false;
-      if (++t >= n) break;
-    }
-    if (rr != 0) {  // the unit's last box had rows to spare
-      rr = 0;
-      release_box();
+    if (lane == 0)
+      for (int i = 0; i < kRing && i < U.nbox; ++i) issue(i, i);
+    float A[4][4], B[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) A[j][k] = 0.0f;
+#pragma unroll 1
+    for (int i = 0; i < U.nbox; i += 2) {
+      if (!block(i, A, B)) return false;
+      if (i + 1 < U.nbox && !block(i + 1, B, A)) return false;
     }
     return true;
   }
@@ -298,36 +283,27 @@ __global__ void __maxnreg__(BIN ? 96 : 128) k_stencil_rows(const __grid_constant
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const StripGeom g = strip_geom(kp.a.in.dtype == HP_F32 ? 4 : 2);
-  const int gw = blockIdx.x * nw + warp, stride = gridDim.x * nw;
-  if (gw >= kp.units) return;
-  Ring R;
-  R.bars = reinterpret_cast<uint64_t*>(base) + warp * kRing;
-  R.slots = base + kBarBytes + warp * kRing * g.slot_bytes;
+  const StripGeom g = strip_geom(F32 || kp.a.in.dtype == HP_F32 ? 4 : 2);
+  const int u = blockIdx.x * nw + warp;
+  if (u >= kp.units) return;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(base) + warp * kRing;
+  unsigned char* const slots = base + kBarBytes + warp * kRing * g.slot_bytes;
   if (lane == 0) {
 #pragma unroll
-    for (int i = 0; i < kRing; ++i) mbar_init(R.bars + i, 1);
+    for (int i = 0; i < kRing; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
   }
   __syncwarp();
-  R.issued = R.released = 0;
-  R.iu = gw;
-  R.ij = 0;
-  R.IU = unit_geom(kp, g, gw);
-  for (int i = 0; i < kRing; ++i) issue_one(kp, g, R, stride, lane);
-  for (int u = gw; u < kp.units; u += stride) {
-    StripRun<F32, EPI, BIN> run(kp, g, R, unit_geom(kp, g, u), lane, stride);
-    if (!run.run()) {
-      // a box never arrived: report, wait (bounded) for the copies still in
-      // flight into this warp's slots, and stop
-      if (lane == 0) {
-        atomicExch(kp.a.err, 1);
-        for (unsigned b = R.released; b < R.issued; ++b)
-          mbar_wait_poll(R.bars + b % kRing, (b / kRing) & 1u, 100000000ull);
-      }
-      __syncwarp();
-      return;
+  const Unit U = unit_geom(kp, g, u);
+  StripRun<F32, EPI, BIN> run(kp, g, U, slots, bars, lane);
+  if (!run.run()) {
+    // a box never arrived: report, and wait (bounded) for copies still in
+    // flight into this warp's slots (a slot's phase is at most one behind)
+    if (lane == 0) {
+      atomicExch(kp.a.err, 1);
+      for (int i = 0; i < kRing; ++i) mbar_wait_poll(bars + i, i < run.s ? run.phase ^ 1 : run.phase, 100000000ull);
     }
+    __syncwarp();
   }
 }
 
@@ -359,14 +335,15 @@ int stencil_rows_strip_w(int in_dtype) { return strip_geom(in_dtype == HP_F32 ? 
 
 int stencil_rows_smem_bytes(int threads, int in_dtype) {
   const StripGeom g = strip_geom(in_dtype == HP_F32 ? 4 : 2);
-  return 128 + kBarBytes + (threads / 32) * kRing * g.slot_bytes;
+  return 2 * 128 + kBarBytes + (threads / 32) * kRing * g.slot_bytes;  // alignment, and room for lane 31's right columns
 }
 
-// Persistent grid: enough CTAs to fill every SM at the kernel's occupancy, or
-// fewer when there are fewer units.
+// CTAs for `units` runs, one per warp; for 1 << 30 units: the CTAs that fill every
+// SM at the kernel's occupancy.
 int stencil_rows_grid(const ChainArgs& a, int units, int threads, int smem_bytes) {
   const int nw = threads / 32;
   const int need = (units + nw - 1) / nw;
+  if (units < 1 << 30) return need;
   int dev = 0, sms = 0, per_sm = 0, variant = 0;
   SRowsKernel kern = pick_kernel(a, &variant);
   if (cudaGetDevice(&dev) != cudaSuccess ||

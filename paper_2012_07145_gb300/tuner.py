@@ -170,7 +170,7 @@ def app_candidates(app, dtype="f32"):
     tiled_w = (32, 64, 96) if app == "harris" else (64, 128)
     for tw, th, t, sy in itertools.product(tiled_w, (16, 32, 64), (128, 256), (4, 8)):
         out.append(dict(schedule="fused", impl=hp.HP_IMPL_AUTO, tile_w=tw, tile_h=th, threads=t, serial_y=sy))
-    runs = (8, 11, 14, 17, 20, 26, 32) if app == "harris" else (12, 16, 20, 24, 32, 48, 64, 96)
+    runs = (8, 11, 14, 17, 20, 26, 32) if app == "harris" else (0, 4, 8, 12, 16, 20, 24, 32, 48, 64, 96)
     strip = 112 if dtype in ("f16", "bf16") else 120      # 2-byte inputs take 112-column strips
     for th, t in itertools.product(runs, (64, 128, 192, 256)):
         out.append(dict(schedule="fused", impl=hp.HP_IMPL_WAVE, tile_w=strip, tile_h=th, threads=t))
@@ -324,7 +324,9 @@ def tune(pipeline, w, h, dtype, quick=False, log=print):
     plain_ms = time_candidate(p, bi, hp.buffer_from_tensor(y, odt), stream, flush)
     log(f"{key(pipeline, w, h, dtype)}: stage-per-kernel {plain_ms:.4f} ms")
     results, pruned = [], []
+    order = {}
     for c in wl["candidates"](quick):
+        order[id(c)] = len(order)
         try:
             wl["apply"](p, ids, c)
             ms, attrs = time_candidate(p, bi, hp.buffer_from_tensor(y, odt), stream, flush, probe=True)
@@ -343,11 +345,12 @@ def tune(pipeline, w, h, dtype, quick=False, log=print):
         log(f"{ms:.4f} ms {c}")
     results.sort(key=lambda r: r[0])
     best = results[0]
-    # event times come in steps of about 2 us: candidates within one step of the
-    # best are told apart by bursts of replays
-    near = [r for r in results if r[0] <= best[0] + 0.0025][:24]
+    # event times come in steps of about 2 us: candidates on the best's step are
+    # told apart by bursts of replays, the first listed within 2% taken
+    near = sorted((r for r in results if r[0] <= best[0] + 0.0006), key=lambda r: order[id(r[1])])[:40]
     if best[0] < 0.05 and len(near) > 1:
-        best = min(near, key=lambda r: burst_ms(wl, p, ids, r[1], bi, hp.buffer_from_tensor(y, odt), stream))
+        bursts = [burst_ms(wl, p, ids, r[1], bi, hp.buffer_from_tensor(y, odt), stream) for r in near]
+        best = next(r for r, ms in zip(near, bursts) if ms <= 1.02 * min(bursts))
     return dict(workload=dict(pipeline=pipeline, w=w, h=h, dtype=dtype), kind=wl["kind"], params=best[1],
                 ms=best[0], plain_ms=plain_ms, registers=best[2], candidates=len(results),
                 pruned_spills=len(pruned), top5=[dict(ms=m, registers=r, **c) for m, c, r in results[:5]],
