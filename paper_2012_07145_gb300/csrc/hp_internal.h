@@ -179,13 +179,20 @@ struct GridArgs {
   ImgView out;   // slice: the 1-channel output
   int s, gz;
   float inv_s, inv_r;
+  int pairs;     // slice: the grid is in pair layout
 };
+
+// Pair layout of a blurred grid that only slices read: [gy][gx][level][2], value
+// and weight of a level together; a cell's levels padded to an even number, so
+// two levels are one aligned 128-bit store.
+HPHD int grid_pair_levels(int gz) { return (gz + 1) & ~1; }
 
 // Blur of a bilateral grid (k_grid.cu): [1,4,6,4,1]/16 along the range levels,
 // then x, then y; rows per run of the streaming kernel.
 struct GridBlurArgs {
   ImgView in, out;
   int gz, rows;
+  int pairs;     // out is in pair layout
 };
 
 // One point-wise stage over f32 images (k_pointwise.cu).

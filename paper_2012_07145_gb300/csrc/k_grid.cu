@@ -63,14 +63,17 @@ __global__ void __launch_bounds__(kSplatThreads) k_grid_splat(const GridArgs a) 
 // The splat of 8 x 8-pixel cells: a block of 4 warps takes 32 consecutive
 // cells of a grid row, lane = cell, warp w = the cell's pixel rows 2w and 2w+1
 // (two 128-bit loads per row for interior cells); each warp accumulates into
-// its own lane-private copy, then the four copies are added in warp order.
+// its own lane-private copy, then the four copies are added in warp order.  The
+// copies take the shared memory of the grid's own range levels (11 KB at 11, not
+// the 32 KB of the most): every block of a 2560x1536 image is resident at once.
 __global__ void __launch_bounds__(128) k_grid_splat8(const GridArgs a) {
   grid_dep_sync();
-  __shared__ float acc[4][2 * kMaxGZ][32];
+  extern __shared__ float accs[];   // [4][2 gz][32]
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float* const acc = accs + w * 2 * a.gz * 32 + lane;
   const int gx = blockIdx.x * 32 + lane, gy = blockIdx.y;
   const bool valid = gx < a.grid.w;
-  for (int j = 0; j < 2 * a.gz; ++j) acc[w][j][lane] = 0.0f;
+  for (int j = 0; j < 2 * a.gz; ++j) acc[j * 32] = 0.0f;
   if (valid) {
     const int W = a.in.w, H = a.in.h;
     const int x0 = gx * 8 - 4;
@@ -92,15 +95,17 @@ __global__ void __launch_bounds__(128) k_grid_splat8(const GridArgs a) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int z = range_level(v[i], a.inv_r, a.gz);
-        acc[w][2 * z][lane] = __fadd_rn(acc[w][2 * z][lane], v[i]);
-        acc[w][2 * z + 1][lane] = __fadd_rn(acc[w][2 * z + 1][lane], 1.0f);
+        acc[2 * z * 32] = __fadd_rn(acc[2 * z * 32], v[i]);
+        acc[(2 * z + 1) * 32] = __fadd_rn(acc[(2 * z + 1) * 32], 1.0f);
       }
     }
   }
   __syncthreads();
   if (!valid) return;
   for (int j = w; j < 2 * a.gz; j += 4) {
-    const float t = __fadd_rn(__fadd_rn(__fadd_rn(acc[0][j][lane], acc[1][j][lane]), acc[2][j][lane]), acc[3][j][lane]);
+    const float* p = accs + j * 32 + lane;
+    const int copy = 2 * a.gz * 32;
+    const float t = __fadd_rn(__fadd_rn(__fadd_rn(p[0], p[copy]), p[2 * copy]), p[3 * copy]);
     reinterpret_cast<float*>((char*)a.grid.data + (long long)j * a.grid.ps + (long long)gy * a.grid.rs)[gx] = t;
   }
 }
@@ -168,6 +173,70 @@ __global__ void __launch_bounds__(256) k_grid_slice(const GridArgs a) {
   }
 }
 
+typedef unsigned long long u64;
+
+__device__ __forceinline__ u64 pack2(float a, float b) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// lerp of (value, weight) at once: b - a and the fused step, each rounded once as in lerp().
+__device__ __forceinline__ u64 lerp2(u64 a, u64 b, float f) {
+  const u64 minus = pack2(-1.0f, -1.0f);
+  return fma2(pack2(f, f), fma2(a, minus, b), a);
+}
+
+// The slice of a grid in pair layout (see grid_pair_levels): a cell's (value,
+// weight) pairs lie together, level by level, so a corner of a pixel's two range
+// levels is two adjacent 64-bit loads instead of four 32-bit ones from four
+// planes, and the pair is interpolated by the paired FP32 instructions.  A warp
+// takes 32 consecutive pixels of 4 rows: at s = 8 a load of the warp touches the
+// levels of 4 cells (a few cache lines), where four pixels of a row per thread
+// touched 16.  SAME: the cell size is a power of two >= 4, so a thread's four
+// pixels (rows 4 q .. 4 q + 3 of a column) lie in one cell.
+template <bool SAME>
+__global__ void __launch_bounds__(256) k_grid_slice_pairs(const GridArgs a) {
+  grid_dep_sync();
+  const int x = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int yb = blockIdx.y * 32 + (threadIdx.x >> 5) * 4;
+  const int W = a.in.w, H = a.in.h;
+  if (x >= W || yb >= H) return;
+  const int gw = a.grid.w, gh = a.grid.h, gzp = grid_pair_levels(a.gz);
+  const float gxf = __fmul_rn((float)x, a.inv_s);
+  const float flx = floorf(gxf), fx = __fsub_rn(gxf, flx);
+  const u64* const c0 = (const u64*)a.grid.data + (long long)iclamp((int)flx, 0, gw - 1) * gzp;
+  const u64* const c1 = (const u64*)a.grid.data + (long long)iclamp((int)flx + 1, 0, gw - 1) * gzp;
+  const int pitch = gw * gzp;   // pairs per grid row
+  float v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = gray_at(a.in, x, imin(yb + k, H - 1));
+  int r0 = 0, r1 = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float gyf = __fmul_rn((float)(yb + k), a.inv_s), gzf = __fmul_rn(v[k], a.inv_r);
+    const float fly = floorf(gyf), flz = floorf(gzf);
+    const float fy = __fsub_rn(gyf, fly), fz = __fsub_rn(gzf, flz);
+    if (!SAME || k == 0) {
+      r0 = iclamp((int)fly, 0, gh - 1) * pitch;
+      r1 = iclamp((int)fly + 1, 0, gh - 1) * pitch;
+    }
+    const int z0 = iclamp((int)flz, 0, a.gz - 1), z1 = iclamp((int)flz + 1, 0, a.gz - 1);
+    const u64 lo = lerp2(lerp2(__ldg(c0 + r0 + z0), __ldg(c1 + r0 + z0), fx),
+                         lerp2(__ldg(c0 + r1 + z0), __ldg(c1 + r1 + z0), fx), fy);
+    const u64 hi = lerp2(lerp2(__ldg(c0 + r0 + z1), __ldg(c1 + r0 + z1), fx),
+                         lerp2(__ldg(c0 + r1 + z1), __ldg(c1 + r1 + z1), fx), fy);
+    float val, wt;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(val), "=f"(wt) : "l"(lerp2(lo, hi, fz)));
+    const float o = wt > 0.0f ? __fdiv_rn(val, wt) : v[k];
+    if (yb + k < H) reinterpret_cast<float*>((char*)a.out.data + (long long)(yb + k) * a.out.rs)[x] = o;
+  }
+}
+
 }  // namespace
 
 int grid_max_levels() { return kMaxGZ; }
@@ -176,7 +245,7 @@ int launch_grid_splat(const GridArgs& a, void* stream) {
   if (a.gz < 1 || a.gz > kMaxGZ || a.s < 1 || a.grid.dtype != HP_F32 || a.grid.c < 2 * a.gz) return (int)cudaErrorInvalidValue;
   if (a.s == 8) {
     dim3 grid8((a.grid.w + 31) / 32, a.grid.h, 1);
-    { const int le_ = launch_kernel(k_grid_splat8, grid8, dim3(128), 0, stream, a); if (le_) return le_; }
+    { const int le_ = launch_kernel(k_grid_splat8, grid8, dim3(128), 4 * 2 * a.gz * 32 * sizeof(float), stream, a); if (le_) return le_; }
   } else {
     dim3 grid((a.grid.w + kSplatThreads - 1) / kSplatThreads, a.grid.h, 1);
     { const int le_ = launch_kernel(k_grid_splat, grid, dim3(kSplatThreads), 0, stream, a); if (le_) return le_; }
@@ -188,7 +257,9 @@ int launch_grid_splat(const GridArgs& a, void* stream) {
 int launch_grid_slice(const GridArgs& a, void* stream) {
   if (a.gz < 1 || a.grid.dtype != HP_F32 || a.out.dtype != HP_F32 || a.grid.c < 2 * a.gz) return (int)cudaErrorInvalidValue;
   dim3 grid((a.in.w + 127) / 128, (a.in.h + 7) / 8, 1);
-  { const int le_ = launch_kernel(k_grid_slice, grid, dim3(256), 0, stream, a); if (le_) return le_; }
+  if (a.pairs) grid = dim3((a.in.w + 31) / 32, (a.in.h + 31) / 32, 1);
+  auto kern = !a.pairs ? k_grid_slice : a.s >= 4 && (a.s & (a.s - 1)) == 0 ? k_grid_slice_pairs<true> : k_grid_slice_pairs<false>;
+  { const int le_ = launch_kernel(kern, grid, dim3(256), 0, stream, a); if (le_) return le_; }
   __atomic_add_fetch(&g_launches, 1ULL, __ATOMIC_RELAXED);
   return (int)cudaGetLastError();
 }
@@ -197,12 +268,13 @@ int launch_grid_slice(const GridArgs& a, void* stream) {
 // ---- the blur of the grid (the group: range-level blur, x blur, y blur) ----
 //
 // k_grid_blur: one warp per strip of 28 grid columns (lanes 0, 1, 30, 31 only
-// feed their neighbours), one of the two halves of a cell (values or weights)
-// and a chunk of 4 range levels, walking down a run of grid rows.  Per row it
-// loads the chunk's levels and two more on each side (clamped), blurs along
-// the levels, then along x (neighbours by warp shuffles); the y blur is five
-// accumulators per level, each fed its taps in order as the rows arrive, so
-// the float operations are those of the three stages one after the other.
+// feed their neighbours) and a chunk of 4 range levels, values and weights,
+// walking down a run of grid rows.  Per row it loads the chunk's levels and two
+// more on each side (clamped), blurs along the levels, then along x (neighbours
+// by warp shuffles); the y blur is five accumulators per level, each fed its taps
+// in order as the rows arrive, so the float operations are those of the three
+// stages one after the other.  Read by slices alone, the result is stored in
+// pair layout (one lane's 4 levels are two 128-bit stores), else in planes.
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
@@ -216,10 +288,10 @@ struct GridBlurParams {
 
 struct BlurRun {
   const GridBlurParams& P;
-  int x, k, z0, y0, nout, T;
+  int x, z0, y0, nout, T;
   bool prod;
-  float acc[kZC][5];
-  float ld[kZC + 4];  // the row's levels z0-2 .. z0+kZC+1 (clamped), in flight
+  float acc[2][kZC][5];
+  float ld[2][kZC + 4];  // the row's levels z0-2 .. z0+kZC+1 (clamped), in flight
 
   __device__ __forceinline__ explicit BlurRun(const GridBlurParams& p) : P(p) {}
 
@@ -230,8 +302,9 @@ struct BlurRun {
     const char* row = (const char*)g.data + (long long)y * g.rs;
 #pragma unroll
     for (int i = 0; i < kZC + 4; ++i) {
-      const int c = 2 * iclamp(z0 - 2 + i, 0, P.a.gz - 1) + k;
-      ld[i] = __ldg(reinterpret_cast<const float*>(row + c * g.ps) + xc);
+      const float* p = reinterpret_cast<const float*>(row + 2 * iclamp(z0 - 2 + i, 0, P.a.gz - 1) * g.ps) + xc;
+      ld[0][i] = __ldg(p);
+      ld[1][i] = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(p) + g.ps));
     }
   }
 
@@ -240,31 +313,47 @@ struct BlurRun {
   // tap 0 starts output t, tap 4 completes output t - 4.
   template <int PH>
   __device__ __forceinline__ void row(int t) {
-    float v[kZC + 4];
+    float v[2][kZC + 4];
 #pragma unroll
-    for (int i = 0; i < kZC + 4; ++i) v[i] = ld[i];
+    for (int i = 0; i < kZC + 4; ++i) { v[0][i] = ld[0][i]; v[1][i] = ld[1][i]; }
     if (t + 1 < T) fetch(t + 1);
     const float w[5] = {0.0625f, 0.25f, 0.375f, 0.25f, 0.0625f};
     const int ofin = t - 4;
     const bool st = prod && ofin >= 0 && ofin < nout;
+    float done[2][kZC];
 #pragma unroll
-    for (int q = 0; q < kZC; ++q) {
-      const float zb = tap5_binomial16(v[q], v[q + 1], v[q + 2], v[q + 3], v[q + 4]);
-      const float l2 = __shfl_up_sync(kFull, zb, 2), l1 = __shfl_up_sync(kFull, zb, 1);
-      const float r1 = __shfl_down_sync(kFull, zb, 1), r2 = __shfl_down_sync(kFull, zb, 2);
-      const float h = tap5(w, l2, l1, zb, r1, r2);
-      // slot of output t - j is (t - j) mod 5 = (PH - j) mod 5
-      float& fin = acc[q][(PH + 1) % 5];                 // output t - 4: tap 4, complete
-      fin = __fmaf_rn(w[4], h, fin);
-      if (st && z0 + q < P.a.gz) {
-        const ImgView& o = P.a.out;
-        reinterpret_cast<float*>((char*)o.data + (long long)(2 * (z0 + q) + k) * o.ps +
-                                 (long long)(y0 + ofin) * o.rs)[x] = fin;
+    for (int q = 0; q < kZC; ++q)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float zb = tap5_binomial16(v[k][q], v[k][q + 1], v[k][q + 2], v[k][q + 3], v[k][q + 4]);
+        const float l2 = __shfl_up_sync(kFull, zb, 2), l1 = __shfl_up_sync(kFull, zb, 1);
+        const float r1 = __shfl_down_sync(kFull, zb, 1), r2 = __shfl_down_sync(kFull, zb, 2);
+        const float h = tap5(w, l2, l1, zb, r1, r2);
+        // slot of output t - j is (t - j) mod 5 = (PH - j) mod 5
+        float (&s)[5] = acc[k][q];
+        done[k][q] = __fmaf_rn(w[4], h, s[(PH + 1) % 5]);        // output t - 4: tap 4, complete
+        s[(PH + 2) % 5] = __fmaf_rn(w[3], h, s[(PH + 2) % 5]);   // output t - 3
+        s[(PH + 3) % 5] = __fmaf_rn(w[2], h, s[(PH + 3) % 5]);   // output t - 2
+        s[(PH + 4) % 5] = __fmaf_rn(w[1], h, s[(PH + 4) % 5]);   // output t - 1
+        s[PH] = __fmul_rn(w[0], h);                              // output t: tap 0
       }
-      acc[q][(PH + 2) % 5] = __fmaf_rn(w[3], h, acc[q][(PH + 2) % 5]);  // output t - 3
-      acc[q][(PH + 3) % 5] = __fmaf_rn(w[2], h, acc[q][(PH + 3) % 5]);  // output t - 2
-      acc[q][(PH + 4) % 5] = __fmaf_rn(w[1], h, acc[q][(PH + 4) % 5]);  // output t - 1
-      acc[q][PH] = __fmul_rn(w[0], h);                                  // output t: tap 0
+    if (!st) return;
+    const ImgView& o = P.a.out;
+    if (P.a.pairs) {
+      const int gzp = grid_pair_levels(P.a.gz);
+      float* p = (float*)o.data + (((long long)(y0 + ofin) * o.w + x) * gzp + z0) * 2;
+#pragma unroll
+      for (int q = 0; q < kZC; q += 2)
+        if (z0 + q < gzp)
+          *reinterpret_cast<float4*>(p + 2 * q) = make_float4(done[0][q], done[1][q], done[0][q + 1], done[1][q + 1]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < kZC; ++q)
+        if (z0 + q < P.a.gz) {
+          char* p = (char*)o.data + (long long)2 * (z0 + q) * o.ps + (long long)(y0 + ofin) * o.rs;
+          reinterpret_cast<float*>(p)[x] = done[0][q];
+          reinterpret_cast<float*>(p + o.ps)[x] = done[1][q];
+        }
     }
   }
 
@@ -273,9 +362,7 @@ struct BlurRun {
     const int strip = u % P.strips;
     int rest = u / P.strips;
     const int zc = rest % P.zchunks;
-    rest /= P.zchunks;
-    k = rest & 1;
-    const int run_idx = rest >> 1;
+    const int run_idx = rest / P.zchunks;
     x = strip * kBlurStrip + lane - 2;
     prod = lane >= 2 && lane < 2 + kBlurStrip && x < P.a.in.w;
     z0 = zc * kZC;
@@ -285,7 +372,7 @@ struct BlurRun {
 #pragma unroll
     for (int q = 0; q < kZC; ++q)
 #pragma unroll
-      for (int s = 0; s < 5; ++s) acc[q][s] = 0.0f;
+      for (int s = 0; s < 5; ++s) acc[0][q][s] = acc[1][q][s] = 0.0f;
     fetch(0);
     for (int t = 0; t < T; t += 5) {
       row<0>(t);
@@ -315,7 +402,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_blur(const GridBlurParams P) {
 int grid_blur_units(const GridBlurArgs& a) {
   const int strips = (a.in.w + kBlurStrip - 1) / kBlurStrip;
   const int zchunks = (a.gz + kZC - 1) / kZC;
-  return strips * zchunks * 2 * ((a.in.h + a.rows - 1) / a.rows);
+  return strips * zchunks * ((a.in.h + a.rows - 1) / a.rows);
 }
 
 int launch_grid_blur(const GridBlurArgs& a, int grid, void* stream) {
@@ -327,7 +414,7 @@ int launch_grid_blur(const GridBlurArgs& a, int grid, void* stream) {
   kp.strips = (a.in.w + kBlurStrip - 1) / kBlurStrip;
   kp.zchunks = (a.gz + kZC - 1) / kZC;
   kp.runs = (a.in.h + a.rows - 1) / a.rows;
-  kp.units = kp.strips * kp.zchunks * 2 * kp.runs;
+  kp.units = kp.strips * kp.zchunks * kp.runs;
   { const int le_ = launch_kernel(k_grid_blur, dim3(grid), dim3(256), 0, stream, kp); if (le_) return le_; }
   __atomic_add_fetch(&g_launches, 1ULL, __ATOMIC_RELAXED);
   return (int)cudaGetLastError();

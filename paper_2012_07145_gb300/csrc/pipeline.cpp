@@ -1254,6 +1254,28 @@ hp_status build_ll_level_rows(const hp_pipeline* p, const Plan& plan, GroupPlan&
   return HP_OK;
 }
 
+// A blurred grid that nothing but slices reads goes to them in pair layout.
+void plan_grid_pairs(const hp_pipeline* p, Plan& plan) {
+  for (GroupPlan& b : plan.groups) {
+    if (b.kernel != HP_KERNEL_GRID_BLUR || b.output == p->output) continue;
+    std::vector<GroupPlan*> slices;
+    bool only = true;
+    for (size_t s = 0; s < p->stages.size(); ++s) {
+      const Stage& st = p->stages[s];
+      if (std::find(st.inputs.begin(), st.inputs.end(), b.output) == st.inputs.end()) continue;
+      GroupPlan* g = nullptr;
+      for (GroupPlan& c : plan.groups)
+        if (c.kernel == HP_KERNEL_GRID_SLICE && c.output == (int)s) g = &c;
+      only = only && g && st.inputs[0] == b.output && st.inputs[1] != b.output && (int)st.params[0] >= 1 &&
+             g->grid.gz == b.gblur.gz;
+      slices.push_back(g);
+    }
+    if (!only) continue;
+    b.gblur.pairs = 1;
+    for (GroupPlan* g : slices) g->grid.pairs = 1;
+  }
+}
+
 hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
   plan.in_dom = in_dom;
   hp_status s = infer_domains(p, in_dom, plan.dom);
@@ -1524,6 +1546,7 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
       return fail(HP_ERR_UNSUPPORTED, "a batch of %d images needs every group on a batch-aware kernel "
                                       "(fused Harris or histogram equalization)", p->batch);
   }
+  plan_grid_pairs(p, plan);
   return HP_OK;
 }
 
@@ -1545,7 +1568,10 @@ hp_status ensure_scratch(hp_pipeline* p, Plan& plan, cudaStream_t stream) {
     if (gp.output == p->output) continue;
     const Stage& st = p->stages[gp.output];
     Scratch sc;
-    sc.bytes = scratch_bytes(st, plan.dom[gp.output]);
+    const Dom d = plan.dom[gp.output];
+    sc.bytes = gp.kernel == HP_KERNEL_GRID_BLUR && gp.gblur.pairs
+                   ? (size_t)d.w * d.h * grid_pair_levels(gp.gblur.gz) * 8
+                   : scratch_bytes(st, d);
     int e = cudaMalloc(&sc.ptr, sc.bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();

@@ -1,0 +1,49 @@
+"""Plan-level choices between a producer and its consumers (GPU): the blurred
+grid handed to slices in pair layout, against a schedule that does not, bit for bit."""
+
+import pytest
+import torch
+
+import __graft_entry__
+from gpu_util import bits, run, to_device
+from paper_2012_07145_gb300 import hp, pipelines, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("h,w", [(1, 1), (5, 33), (64, 96), (131, 257), (200, 31)])
+@pytest.mark.parametrize("s,r", [(1, 0.5), (4, 0.2), (8, 0.1), (12, 0.1), (16, 0.05), (3, 0.04)])
+def test_grid_pairs(h, w, s, r):
+    """Cells of powers of two and others, even and odd level counts, images of
+    less than a block; a plan per size of one pipeline."""
+    img = synth.gray_f32_gradient_noise(h, w, seed=h + w)
+    img[0, ::3, ::5] = 1.0    # the last range level
+    x = to_device(img, hp.HP_F32)
+    p = pipelines.bilateral_grid(s, r)
+    plain = run(p, [x], [hp.HP_F32], (1, h, w), hp.HP_F32)
+    pipelines.bilateral_grid_fused_schedule(p)
+    for _ in range(2):
+        assert torch.equal(bits(run(p, [x], [hp.HP_F32], (1, h, w), hp.HP_F32)), bits(plain))
+
+
+def test_grid_read_by_more_than_slices_stays_planar():
+    """The blurred grid is the output itself: written in planes."""
+    F = hp.HP_F32
+    h, w, s, r, gz = 70, 90, 8, 0.1, 11
+    x = to_device(synth.gray_f32_gradient_noise(h, w, seed=2), F)
+    outs = []
+    for fused in (False, True):
+        p = hp.Pipeline([F], [1])
+        g = p.add_stage(hp.HP_GRID_SPLAT, [p.input(0)], 2 * gz, F, params=[s, r])
+        bz = p.add_stage(hp.HP_POINTWISE, [g], 2 * gz, F, op=hp.HP_OP_ZBLUR, params=[gz])
+        bx = p.add_stage(hp.HP_STENCIL, [bz], 2 * gz, F, rx=2, ry=0, wx=pipelines.BINOMIAL16, wy=[1.0])
+        p.set_output(p.add_stage(hp.HP_STENCIL, [bx], 2 * gz, F, rx=0, ry=2, wx=[1.0], wy=pipelines.BINOMIAL16))
+        if fused:
+            p.schedule([0, 1, 1, 1])
+        outs.append(run(p, [x], [F], (2 * gz, 10, 13), F))
+    assert torch.equal(bits(outs[0]), bits(outs[1]))
