@@ -169,6 +169,7 @@ struct MaxArgs {
 struct InterpArgs {
   ImgView fine, coarse, out;  // D_l (4 ch), I_{l+1} (4 ch), the group's output
   int rows, threads, final_div, vec;
+  int premul;                 // fine is the image before its premultiply
   int* err;  // device error word (bounded waits)
 };
 
@@ -235,6 +236,7 @@ struct HarrisArgs {
 struct LLDownArgs {
   ImgView src, out;
   int C;                       // channels produced
+  int premul;                  // src is an RGBA image before its premultiply (C = 4)
   int remap;
   float gray_scale, sigma, alpha, beta;
   int K;
@@ -322,8 +324,8 @@ int ll_remap_rows_ok(const LLDownArgs& a, int in_dtype);
 int ll_remap_rows_grid(int in_dtype, int units, int threads);
 int launch_ll_remap_rows(const LLDownArgs& a, int rows, int threads, int grid, void* stream);
 int ll_down_rows_ok(const LLDownArgs& a, int src_dtype);
-int ll_down_rows_groups(int C);
-int ll_down_rows_grid(int C, int units, int threads);
+int ll_down_rows_groups(int C, int premul);
+int ll_down_rows_grid(int C, int premul, int units, int threads);
 int launch_ll_down_rows(const LLDownArgs& a, int rows, int threads, int grid, void* stream);
 int ll_level_rows_strip_w();
 int ll_level_rows_ok(const LLLevelArgs& a);

@@ -46,70 +46,30 @@ struct InterpParams {
   int strips, units;
 };
 
-// The warp's ring: box q (in issue order, which is the order of use) lives in
-// slot q % kRing and completes phase (q / kRing) & 1 of that slot's mbarrier.
-// Box j of a run holds fine rows 2 (n0 + j) and 2 (n0 + j) + 1.
-struct Ring {
-  unsigned char* slots;
-  uint64_t* bars;
-  unsigned issued, released;
-  int iu, ij, inrun, ix, iy;  // next box: unit, box within it, the unit's boxes, its fine origin
-};
-
-__device__ __forceinline__ void set_unit(const InterpParams& P, Ring& R) {
-  const int strip = R.iu % P.strips, run = R.iu / P.strips;
-  const int n0 = run * P.a.rows;
-  R.inrun = imin(P.a.rows, P.a.coarse.h - n0);
-  R.ix = 2 * (strip * kStripW) - 4;
-  R.iy = 2 * n0;
-}
-
-__device__ __forceinline__ void issue_one(const InterpParams& P, Ring& R, int stride, int lane) {
-  if (R.iu >= P.units) return;
-  if (lane == 0) {
-    const int s = R.issued % kRing;
-    // the warp's reads of this slot (its previous box) come before the copy
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive_expect_tx(R.bars + s, (unsigned)kBoxBytes);
-    tma_load_3d(R.slots + s * kSlotBytes, &P.tmap, R.ix, R.iy + 2 * R.ij, 0, R.bars + s);
-  }
-  ++R.issued;
-  if (++R.ij == R.inrun) {
-    R.ij = 0;
-    R.iu += stride;
-    if (R.iu < P.units) set_unit(P, R);
-  }
-}
-
-template <bool FINAL>
+// One run of coarse rows of one strip.  Box j (fine rows 2 (n0 + j) and
+// 2 (n0 + j) + 1) lives in slot j % kRing of the warp's ring and completes phase
+// (j / kRing) & 1 of that slot's mbarrier.  PREMUL: the fine image is not yet
+// premultiplied (the premultiply stage is folded in).
+template <bool FINAL, bool PREMUL>
 struct InterpRun {
   const InterpParams& P;
-  Ring& R;
-  const int stride;
+  unsigned char* const slots;
+  uint64_t* const bars;
   int m, cm, X0, X1, n0, nrun, c0, c1;  // c0, c1: X0, X1 as columns of the box
   bool pair, prod, ok1;
-  unsigned q;                 // box being read
-  const float* box;           // its slot
+  int s, phase;               // slot and phase of the next box
+  const float* box;           // the box being read
   float hx[3][4][2];  // x-passed coarse rows (window slot, channel, fine column)
   float raw[4];       // the next coarse row, in flight
 
-  __device__ __forceinline__ InterpRun(const InterpParams& p, Ring& r, int stride_)
-      : P(p), R(r), stride(stride_), q(r.released), box(nullptr) {}
+  __device__ __forceinline__ InterpRun(const InterpParams& p, unsigned char* slots_, uint64_t* bars_)
+      : P(p), slots(slots_), bars(bars_), s(0), phase(0), box(nullptr) {}
 
-  __device__ __forceinline__ bool wait_box(int lane) {
-    int ok = 1;
-    if (lane == 0) ok = mbar_wait_poll(R.bars + q % kRing, (q / kRing) & 1u, 2000000000ull);
-    __syncwarp();
-    ok = __shfl_sync(kFull, ok, 0);
-    box = reinterpret_cast<const float*>(R.slots + (q % kRing) * kSlotBytes);
-    return ok != 0;
-  }
-
-  __device__ __forceinline__ void release_box(int lane) {
-    ++q;
-    __syncwarp();
-    R.released = q;
-    issue_one(P, R, stride, lane);
+  __device__ __forceinline__ void issue(int strip, int j, int slot) const {
+    // the warp's reads of this slot (its previous box) come before the copy
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive_expect_tx(bars + slot, (unsigned)kBoxBytes);
+    tma_load_3d(slots + slot * kSlotBytes, &P.tmap, 2 * (strip * kStripW) - 4, 2 * (n0 + j), 0, bars + slot);
   }
 
   __device__ __forceinline__ void load_raw(int q) {
@@ -147,6 +107,13 @@ struct InterpRun {
         d[ch][1] = q[c1];
       }
     }
+    if (PREMUL) {
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch) {
+        d[ch][0] = op_premul(d[ch][0], d[3][0], ch);
+        d[ch][1] = op_premul(d[ch][1], d[3][1], ch);
+      }
+    }
     float o[4][2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -178,15 +145,20 @@ struct InterpRun {
 
   // False: a box never arrived.
   template <int PH>
-  __device__ __forceinline__ bool step(int i, int lane) {
+  __device__ __forceinline__ bool step(int strip, int i, int lane) {
     constexpr int A = PH, B = (PH + 1) % 3, C = (PH + 2) % 3;
     xpass<C>();
     if (i + 3 <= nrun + 1) load_raw(i + 3);
-    if (!wait_box(lane)) return false;
+    // every lane waits for the box itself (usually there: one test)
+    if (!__all_sync(kFull, mbar_try_wait(bars + s, phase) || mbar_wait_poll(bars + s, phase, 2000000000ull))) return false;
+    box = reinterpret_cast<const float*>(slots + s * kSlotBytes);
     const int Y = 2 * (n0 + i);
     emit<false, A, B, C>(Y);
     if (Y + 1 < P.a.fine.h) emit<true, A, B, C>(Y + 1);
-    release_box(lane);
+    __syncwarp();   // every lane has read the box
+    if (lane == 0 && i + kRing < nrun) issue(strip, i + kRing, s);
+    phase ^= s == kRing - 1;
+    s = s == kRing - 1 ? 0 : s + 1;
     return true;
   }
 
@@ -204,62 +176,58 @@ struct InterpRun {
     ok1 = prod && 2 * m + 1 <= W - 1;
     n0 = run_idx * P.a.rows;
     nrun = imin(P.a.rows, P.a.coarse.h - n0);
+    if (lane == 0)
+      for (int j = 0; j < kRing && j < nrun; ++j) issue(strip, j, j);
     load_raw(0);
     xpass<0>();
     load_raw(1);
     xpass<1>();
     load_raw(2);
     for (int i = 0; i < nrun; i += 3) {
-      if (!step<0>(i, lane)) return false;
+      if (!step<0>(strip, i, lane)) return false;
       if (i + 1 >= nrun) break;
-      if (!step<1>(i + 1, lane)) return false;
+      if (!step<1>(strip, i + 1, lane)) return false;
       if (i + 2 >= nrun) break;
-      if (!step<2>(i + 2, lane)) return false;
+      if (!step<2>(strip, i + 2, lane)) return false;
     }
     return true;
   }
 };
 
-template <bool FINAL>
+template <bool FINAL, bool PREMUL>
 __global__ void __launch_bounds__(256, 3) k_interp_rows(const __grid_constant__ InterpParams P) {
   grid_dep_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int gw = blockIdx.x * nw + warp, stride = gridDim.x * nw;
-  if (gw >= P.units) return;
-  Ring R;
-  R.bars = reinterpret_cast<uint64_t*>(base) + warp * kRing;
-  R.slots = base + kBarBytes + warp * kRing * kSlotBytes;
+  const int u = blockIdx.x * nw + warp;
+  if (u >= P.units) return;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(base) + warp * kRing;
+  unsigned char* const slots = base + kBarBytes + warp * kRing * kSlotBytes;
   if (lane == 0) {
 #pragma unroll
-    for (int i = 0; i < kRing; ++i) mbar_init(R.bars + i, 1);
+    for (int i = 0; i < kRing; ++i) mbar_init(bars + i, 1);
     fence_mbar_init();
   }
   __syncwarp();
-  R.issued = R.released = 0;
-  R.iu = gw;
-  R.ij = 0;
-  set_unit(P, R);
-  for (int i = 0; i < kRing; ++i) issue_one(P, R, stride, lane);
-  for (int u = gw; u < P.units; u += stride) {
-    InterpRun<FINAL> r(P, R, stride);
-    if (!r.run(u % P.strips, u / P.strips)) {
-      // a box never arrived: report, wait (bounded) for the copies still in
-      // flight into this warp's slots, and stop
-      if (lane == 0) {
-        atomicExch(P.a.err, 1);
-        for (unsigned b = R.released; b < R.issued; ++b) mbar_wait_poll(R.bars + b % kRing, (b / kRing) & 1u, 100000000ull);
-      }
-      __syncwarp();
-      return;
+  InterpRun<FINAL, PREMUL> r(P, slots, bars);
+  if (!r.run(u % P.strips, u / P.strips)) {
+    // a box never arrived: report, and wait (bounded) for copies still in
+    // flight into this warp's slots (a slot's phase is at most one behind)
+    if (lane == 0) {
+      atomicExch(P.a.err, 1);
+      for (int i = 0; i < kRing; ++i) mbar_wait_poll(bars + i, i < r.s ? r.phase ^ 1 : r.phase, 100000000ull);
     }
+    __syncwarp();
   }
 }
 
 typedef void (*InterpKernel)(InterpParams);
 
-InterpKernel pick_kernel(const InterpArgs& a) { return a.final_div ? k_interp_rows<true> : k_interp_rows<false>; }
+InterpKernel pick_kernel(const InterpArgs& a) {
+  if (a.premul) return a.final_div ? k_interp_rows<true, true> : k_interp_rows<false, true>;
+  return a.final_div ? k_interp_rows<true, false> : k_interp_rows<false, false>;
+}
 
 }  // namespace
 
@@ -267,9 +235,12 @@ int interp_rows_strip_w() { return kStripW; }
 
 int interp_rows_smem_bytes(int threads) { return 128 + kBarBytes + (threads / 32) * kRing * kSlotBytes; }
 
+// CTAs for `units` runs, one per warp; for 1 << 30 units: the CTAs that fill every
+// SM at the kernel's occupancy.
 int interp_rows_grid(const InterpArgs& a, int units, int threads) {
   const int nw = threads / 32;
   const int need = (units + nw - 1) / nw;
+  if (units < 1 << 30) return need;
   int dev = 0, sms = 0, per_sm = 0;
   const InterpKernel kern = pick_kernel(a);
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||

@@ -227,8 +227,9 @@ struct RemapRun {
 };
 
 // The plane source: CG channels (from channel c0) of a stack of f32 planes.
-// F32S: the output stored as f32.
-template <int CG, bool F32S>
+// F32S: the output stored as f32.  PREMUL (CG = 4): the source is an RGBA image
+// still to be premultiplied (the premultiply stage is folded in).
+template <int CG, bool F32S, bool PREMUL>
 struct PlaneRun {
   const LLRowsParams& P;
   RunGeom G;
@@ -262,6 +263,13 @@ struct PlaneRun {
     if (t + 2 < G.T) fetch(nxt2, t + 2);
     const int ofin = (t >> 1) - 2;
     const bool st = (PH & 1) == 0 && G.prod && ofin >= 0 && ofin < G.nout;
+    if (PREMUL) {
+#pragma unroll
+      for (int c = 0; c < CG - 1; ++c) {
+        cur[c].x = op_premul(cur[c].x, cur[CG - 1].x, c);
+        cur[c].y = op_premul(cur[c].y, cur[CG - 1].y, c);
+      }
+    }
 #pragma unroll
     for (int c = 0; c < CG; ++c) {
       const float fin = ytaps<PH>(acc[c], xpass(cur[c].x, cur[c].y));
@@ -301,14 +309,14 @@ __global__ void __launch_bounds__(256, 2) k_ll_remap_rows(const LLRowsParams P) 
 }
 
 // One level down of C f32 planes, CG channels per warp unit.
-template <int CG, bool F32S>
+template <int CG, bool F32S, bool PREMUL = false>
 __global__ void __launch_bounds__(256, 2) k_ll_down_rows(const LLRowsParams P) {
   grid_dep_wait();
   const int groups = P.a.C / CG;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < P.units; u += nw) {
     const int rest = u / P.strips;
-    PlaneRun<CG, F32S> r(P);
+    PlaneRun<CG, F32S, PREMUL> r(P);
     r.run(u % P.strips, rest / groups, rest % groups);
   }
 }
@@ -317,13 +325,14 @@ typedef void (*RemapKernel)(LLRowsParams);
 
 // Three channels per unit where the count allows (nine would hold 27
 // accumulators and 54 prefetched values per lane, past the register budget).
-RemapKernel pick_down_kernel(int C, bool f32s) {
+RemapKernel pick_down_kernel(int C, bool f32s, bool premul) {
+  if (premul) return f32s ? k_ll_down_rows<4, true, true> : k_ll_down_rows<4, false, true>;
   static const RemapKernel ks[4] = {k_ll_down_rows<1, false>, k_ll_down_rows<1, true>, k_ll_down_rows<3, false>,
                                     k_ll_down_rows<3, true>};
   return ks[(C % 3 == 0 ? 2 : 0) + (f32s ? 1 : 0)];
 }
 
-int down_group(int C) { return C % 3 == 0 ? 3 : 1; }
+int down_group(int C, bool premul) { return premul ? 4 : C % 3 == 0 ? 3 : 1; }
 
 int resident_ctas(RemapKernel kern, int threads, int need) {
   int dev = 0, sms = 0, per_sm = 0;
@@ -372,25 +381,25 @@ int ll_remap_rows_grid(int in_dtype, int units, int threads) {
 // per warp unit).
 int ll_down_rows_ok(const LLDownArgs& a, int src_dtype) { return !a.remap && src_dtype == HP_F32 && a.C >= 1; }
 
-int ll_down_rows_groups(int C) { return C / down_group(C); }
+int ll_down_rows_groups(int C, int premul) { return C / down_group(C, premul); }
 
-int ll_down_rows_grid(int C, int units, int threads) {
+int ll_down_rows_grid(int C, int premul, int units, int threads) {
   const int nw = threads / 32;
-  return resident_ctas(pick_down_kernel(C, true), threads, (units + nw - 1) / nw);
+  return resident_ctas(pick_down_kernel(C, true, premul), threads, (units + nw - 1) / nw);
 }
 
 int launch_ll_down_rows(const LLDownArgs& a, int rows, int threads, int grid, void* stream) {
-  if (a.src.dtype != HP_F32 || a.remap) return (int)cudaErrorInvalidValue;
+  if (a.src.dtype != HP_F32 || a.remap || (a.premul && a.C != 4)) return (int)cudaErrorInvalidValue;
   if (rows < 1 || threads < 32 || threads > 256 || threads % 32 || grid < 1) return (int)cudaErrorInvalidValue;
   LLRowsParams kp;
   memset(&kp, 0, sizeof kp);
   kp.a = a;
   kp.strips = (a.out.w + kStripW - 1) / kStripW;
   kp.rows = rows;
-  kp.units = kp.strips * ll_down_rows_groups(a.C) * ((a.out.h + rows - 1) / rows);
+  kp.units = kp.strips * ll_down_rows_groups(a.C, a.premul) * ((a.out.h + rows - 1) / rows);
   kp.vec = ((long long)(size_t)a.src.data % 8 == 0) && a.src.rs % 8 == 0 && a.src.ps % 8 == 0;
   const bool f32s = a.st_out == HP_F32 && a.out.dtype == HP_F32;
-  { const int le_ = launch_kernel(pick_down_kernel(a.C, f32s), dim3(grid), dim3(threads), 0, stream, kp); if (le_) return le_; }
+  { const int le_ = launch_kernel(pick_down_kernel(a.C, f32s, a.premul), dim3(grid), dim3(threads), 0, stream, kp); if (le_) return le_; }
   __atomic_add_fetch(&g_launches, 1ULL, __ATOMIC_RELAXED);
   return (int)cudaGetLastError();
 }

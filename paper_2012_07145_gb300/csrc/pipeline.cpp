@@ -106,6 +106,8 @@ struct GroupPlan {
   GridBlurArgs gblur{};
   LLRoles llroles{};
   std::unique_ptr<GPlan> gplan;
+  bool rows_given = false;    // the schedule sets the rows per run
+  bool folded = false;        // computed inside its consumers: no launch, no buffer
   std::vector<int> ext_refs;  // generic: external refs (stage id or -1-k)
   size_t aux_bytes = 0;       // kernel state kept across launches (zeroed once at allocation)
   void* aux = nullptr;
@@ -1135,8 +1137,10 @@ hp_status build_down(const hp_pipeline* p, const Plan& plan, GroupPlan& gp) {
 // about one run per resident warp; the plane kernel, light per row, down to
 // one row so that small levels still spread over the SMs).
 hp_status build_ll_rows(const hp_pipeline* p, const Plan& plan, GroupPlan& gp) {
+  const int premul = gp.lldown.premul;
   down_common_args(p, gp);
   LLDownArgs& a = gp.lldown;
+  a.premul = premul;
   const bool remap = gp.kernel == HP_KERNEL_LL_REMAP_ROWS;
   const int src_dt = stage_dtype_of_ref(p, gp.ext_refs[0]);
   if (remap ? !ll_remap_rows_ok(a, src_dt) : !ll_down_rows_ok(a, src_dt))
@@ -1150,9 +1154,9 @@ hp_status build_ll_rows(const hp_pipeline* p, const Plan& plan, GroupPlan& gp) {
   Dom od = plan.dom[gp.output];
   a.tile_w = gp.tile_w;
   a.tiles_x = (od.w + a.tile_w - 1) / a.tile_w;
-  const int units_per_row = a.tiles_x * (remap ? 1 : ll_down_rows_groups(a.C));
+  const int units_per_row = a.tiles_x * (remap ? 1 : ll_down_rows_groups(a.C, a.premul));
   auto grid_for = [&](int units) {
-    return remap ? ll_remap_rows_grid(src_dt, units, gp.threads) : ll_down_rows_grid(a.C, units, gp.threads);
+    return remap ? ll_remap_rows_grid(src_dt, units, gp.threads) : ll_down_rows_grid(a.C, a.premul, units, gp.threads);
   };
   if (gp.tile_h == 0) {
     const long long warps = (long long)grid_for(1 << 30) * (gp.threads / 32);
@@ -1254,6 +1258,44 @@ hp_status build_ll_level_rows(const hp_pipeline* p, const Plan& plan, GroupPlan&
   return HP_OK;
 }
 
+// A premultiply stage that only streaming interpolate levels (as their fine
+// image) and streaming 4-channel downsamples read is recomputed in them: one
+// multiplication per value, instead of writing and reading the whole premultiplied
+// image (2560x1536 RGBA f32: 63 MB each way and a launch of 17 us).
+hp_status plan_premul_fold(hp_pipeline* p, Plan& plan) {
+  for (GroupPlan& m : plan.groups) {
+    if (m.kernel != HP_KERNEL_PW_ROWS || m.pw.op != HP_OP_PREMUL || m.output == p->output) continue;
+    std::vector<GroupPlan*> users;
+    bool ok = true;
+    for (GroupPlan& g : plan.groups) {
+      if (&g == &m) continue;
+      bool reads = false;
+      for (int s : g.members)
+        for (int r : p->stages[s].inputs) reads = reads || r == m.output;
+      if (!reads) continue;
+      const bool fine = g.kernel == HP_KERNEL_INTERP_ROWS && g.ext_refs[0] == m.output && g.ext_refs[1] != m.output;
+      const bool down = g.kernel == HP_KERNEL_LL_DOWN_ROWS && g.ext_refs[0] == m.output && g.lldown.C == 4;
+      ok = ok && (fine || down);
+      users.push_back(&g);
+    }
+    if (!ok || users.empty()) continue;
+    m.folded = true;
+    for (GroupPlan* g : users) {
+      const int h = g->tile_h;
+      if (g->kernel == HP_KERNEL_INTERP_ROWS) {
+        g->interp.premul = 1;
+      } else {
+        g->lldown.premul = 1;
+        const bool chosen = h != 0 && !g->rows_given;
+        g->tile_h = chosen ? 0 : h;
+        if (hp_status s = build_ll_rows(p, plan, *g)) return s;
+      }
+      g->ext_refs[0] = m.ext_refs[0];
+    }
+  }
+  return HP_OK;
+}
+
 // A blurred grid that nothing but slices reads goes to them in pair layout.
 void plan_grid_pairs(const hp_pipeline* p, Plan& plan) {
   for (GroupPlan& b : plan.groups) {
@@ -1349,6 +1391,7 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
               gp.kernel = remap_ok ? HP_KERNEL_LL_REMAP_ROWS : HP_KERNEL_LL_DOWN_ROWS;
               gp.tile_w = sw;
               gp.tile_h = pick(p->tile_h, g, 0);
+              gp.rows_given = gp.tile_h != 0;
               gp.threads = pick(p->threads, g, 256);
               s = build_ll_rows(p, plan, gp);
               break;
@@ -1547,7 +1590,7 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
                                       "(fused Harris or histogram equalization)", p->batch);
   }
   plan_grid_pairs(p, plan);
-  return HP_OK;
+  return plan_premul_fold(p, plan);
 }
 
 // First realize of a plan: its buffers.  Kernel state is cleared on the
@@ -1565,7 +1608,7 @@ hp_status ensure_scratch(hp_pipeline* p, Plan& plan, cudaStream_t stream) {
     }
   }
   for (const GroupPlan& gp : plan.groups) {
-    if (gp.output == p->output) continue;
+    if (gp.output == p->output || gp.folded) continue;
     const Stage& st = p->stages[gp.output];
     Scratch sc;
     const Dom d = plan.dom[gp.output];
@@ -1678,6 +1721,7 @@ hp_status run_groups(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, const 
 
 hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, const hp_buffer* output, void* stream) {
   for (GroupPlan& gp : plan.groups) {
+    if (gp.folded) continue;
     ImgView out = ref_view(p, plan, gp.output, inputs, output);
     int e = 0;
     switch (gp.kernel) {

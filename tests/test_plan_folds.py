@@ -1,5 +1,6 @@
 """Plan-level choices between a producer and its consumers (GPU): the blurred
-grid handed to slices in pair layout, against a schedule that does not, bit for bit."""
+grid handed to slices in pair layout, and the premultiply recomputed in its
+consumers, each against a schedule that does neither, bit for bit."""
 
 import pytest
 import torch
@@ -47,3 +48,23 @@ def test_grid_read_by_more_than_slices_stays_planar():
             p.schedule([0, 1, 1, 1])
         outs.append(run(p, [x], [F], (2 * gz, 10, 13), F))
     assert torch.equal(bits(outs[0]), bits(outs[1]))
+
+
+@pytest.mark.parametrize("h,w,levels", [(3, 2, 2), (37, 53, 4), (130, 258, 5), (257, 131, 7)])
+def test_premultiply_fold(h, w, levels):
+    """Folded into the first downsample and the finest level; not folded where
+    the finest level runs on the generic kernel."""
+    x = to_device(synth.rgba_sparse_f32(h, w, seed=h), hp.HP_F32)
+    p, ids = pipelines.interpolate(levels)
+    plain = run(p, [x], [hp.HP_F32], (3, h, w), hp.HP_F32)
+    pipelines.interpolate_fused_schedule(p, ids)
+    groups = p.group_count()
+    n0 = hp.launch_count()
+    y = run(p, [x], [hp.HP_F32], (3, h, w), hp.HP_F32)
+    assert hp.launch_count() - n0 == groups - 1
+    assert torch.equal(bits(y), bits(plain))
+    pipelines.interpolate_fused_schedule(p, ids, impl=hp.HP_IMPL_GENERIC)
+    n0 = hp.launch_count()
+    y = run(p, [x], [hp.HP_F32], (3, h, w), hp.HP_F32)
+    assert hp.launch_count() - n0 == p.group_count()
+    assert torch.equal(bits(y), bits(plain))
