@@ -402,8 +402,8 @@ __global__ void __launch_bounds__(256) k_harris_rows(const __grid_constant__ Row
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int esize = kp.a.in.dtype == HP_F32 ? 4 : 2;
   const StripGeom g = strip_geom(esize);
-  const int gw = blockIdx.x * nw + warp, stride = gridDim.x * nw;
-  if (gw >= kp.units) return;
+  const int u = blockIdx.x * nw + warp;
+  if (u >= kp.units) return;
   uint64_t* bars = reinterpret_cast<uint64_t*>(base) + warp * kRing;
   unsigned char* slots = base + kBarBytes + warp * kRing * g.slot_bytes;
   if (lane == 0) {
@@ -412,72 +412,57 @@ __global__ void __launch_bounds__(256) k_harris_rows(const __grid_constant__ Row
     fence_mbar_init();
   }
   __syncwarp();
+  const Unit U = unit_geom(kp, g, u);
+  if (lane == 0)
+    for (int j = 0; j < kRing && j < U.nbox; ++j) issue_box(&kp.tmap, slots, bars, g.slot_bytes, j, U, j);
   HarrisRun<RND, ODT, SPEC> R(kp.a);
   const int W = kp.a.in.w, H = kp.a.in.h;
   R.H = H;
-  unsigned qbase = 0;  // boxes this warp has issued before the current unit
-  for (int u = gw; u < kp.units; u += stride) {
-    const Unit U = unit_geom(kp, g, u);
-    if (lane == 0)
-      for (int j = 0; j < kRing && j < U.nbox; ++j) issue_box(&kp.tmap, slots, bars, g.slot_bytes, qbase + j, U, j);
-    const int c0 = U.x0 + 4 * lane;
-    R.y0 = U.y0;
-    R.top = U.y0 == 0;
-    R.e.left = c0 == 0;
+  const int c0 = U.x0 + 4 * lane;
+  R.y0 = U.y0;
+  R.top = U.y0 == 0;
+  R.e.left = c0 == 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) R.e.right[k] = c0 + k == W - 1;
-    const bool he = U.x0 < 0 || U.x0 + 128 > W;
-    const bool mine = lane >= g.halo_lanes && lane < 32 - g.halo_lanes;
-    const bool st_full = mine && c0 + 3 < kp.a.out.w && ODT != 3;
-    const bool st_part = mine && c0 < kp.a.out.w && !st_full;
-    char* out_row = (char*)kp.a.out.data + (long long)U.img * kp.a.out.ps + (long long)U.oy * kp.a.out.rs;
-    const int n = U.n_steps;
-    const int t_store = U.oy - U.y0 + 2;          // first step whose output row is the run's
-    const int t_edge = H - U.y0;                   // from this step on the gray row lies below the image
-    const int t_top = R.top ? 1 : -1;              // steps 0 .. t_top: gray row 0 or 1 of a top run
-    int failed = 0;
+  for (int k = 0; k < 4; ++k) R.e.right[k] = c0 + k == W - 1;
+  const bool he = U.x0 < 0 || U.x0 + 128 > W;
+  const bool mine = lane >= g.halo_lanes && lane < 32 - g.halo_lanes;
+  const bool st_full = mine && c0 + 3 < kp.a.out.w && ODT != 3;
+  const bool st_part = mine && c0 < kp.a.out.w && !st_full;
+  char* out_row = (char*)kp.a.out.data + (long long)U.img * kp.a.out.ps + (long long)U.oy * kp.a.out.rs;
+  const int n = U.n_steps;
+  const int t_store = U.oy - U.y0 + 2;          // first step whose output row is the run's
+  const int t_edge = H - U.y0;                   // from this step on the gray row lies below the image
+  const int t_top = R.top ? 1 : -1;              // steps 0 .. t_top: gray row 0 or 1 of a top run
 #pragma unroll 1
-    for (int j = 0; kBoxRows * j < n; ++j) {
-      const int t0 = kBoxRows * j;
-      const unsigned char* slot = nullptr;
-      if (t0 < U.n_in) {
-        const unsigned q = qbase + j;
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait_poll(bars + q % kRing, (q / kRing) & 1u, 2000000000ull);
-        ok = __shfl_sync(kFull, ok, 0);
-        if (!ok) {
-          failed = 1;
-          break;
+  for (int j = 0; kBoxRows * j < n; ++j) {
+    const int t0 = kBoxRows * j;
+    const unsigned char* slot = slots + (j % kRing) * g.slot_bytes + lane * 4 * esize;
+    if (t0 < U.n_in) {
+      // every lane waits for the box itself (usually there: one test)
+      const unsigned ph = (j / kRing) & 1u;
+      if (!__all_sync(kFull, mbar_try_wait(bars + j % kRing, ph) || mbar_wait_poll(bars + j % kRing, ph, 2000000000ull))) {
+        // a box never arrived: report, wait (bounded) for the copies still in
+        // flight into this warp's slots, and stop
+        if (lane == 0) {
+          atomicExch(kp.a.err, 1);
+          for (int q = j; q < j + kRing && q < U.nbox; ++q)
+            mbar_wait_poll(bars + q % kRing, (q / kRing) & 1u, 100000000ull);
         }
-        slot = slots + (q % kRing) * g.slot_bytes + lane * 4 * esize;
-      }
-      const bool edge = t0 <= t_top || t0 + kBoxRows - 1 >= t_edge || t0 + kBoxRows > n;
-      if (edge) {
-        if (he) box_steps<true, true>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
-        else box_steps<true, false>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
-      } else {
-        if (he) box_steps<false, true>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
-        else box_steps<false, false>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
-      }
-      if (j + kRing < U.nbox) {  // this box's slot is read: refill it
         __syncwarp();
-        if (lane == 0) issue_box(&kp.tmap, slots, bars, g.slot_bytes, qbase + j + kRing, U, j + kRing);
+        return;
       }
     }
-    if (failed) {
-      // a box never arrived: report, wait (bounded) for the copies still in
-      // flight into this warp's slots, and stop
-      if (lane == 0) {
-        atomicExch(kp.a.err, 1);
-        for (int j = 0; j < U.nbox; ++j) {
-          const unsigned q = qbase + j;
-          mbar_wait_poll(bars + q % kRing, (q / kRing) & 1u, 100000000ull);
-        }
-      }
-      __syncwarp();
-      return;
+    const bool edge = t0 <= t_top || t0 + kBoxRows - 1 >= t_edge || t0 + kBoxRows > n;
+    if (edge) {
+      if (he) box_steps<true, true>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
+      else box_steps<true, false>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
+    } else {
+      if (he) box_steps<false, true>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
+      else box_steps<false, false>(R, t0, n, slot, kp.a.in.dtype, esize, t_store, out_row, c0, st_full, st_part, U, kp.a.out);
     }
-    qbase += U.nbox;
+    __syncwarp();
+    if (lane == 0 && j + kRing < U.nbox)  // this box's slot is read: refill it
+      issue_box(&kp.tmap, slots, bars, g.slot_bytes, j + kRing, U, j + kRing);
   }
 }
 
@@ -527,11 +512,12 @@ int harris_rows_smem_bytes(int threads, int in_dtype) {
   return 128 + kBarBytes + (threads / 32) * kRing * g.slot_bytes;
 }
 
-// Persistent grid: enough CTAs to fill every SM at the kernel's occupancy, or
-// fewer when there are fewer units.
+// CTAs for `units` runs, one per warp; for 1 << 30 units: the CTAs that fill every
+// SM at the kernel's occupancy.
 int harris_rows_grid(const HarrisArgs& a, int units, int threads, int smem_bytes) {
   const int nw = threads / 32;
   const int need = (units + nw - 1) / nw;
+  if (units < 1 << 30) return need;
   int dev = 0, sms = 0, per_sm = 0, variant = 0;
   RowsKernel kern = pick_kernel(a, &variant);
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
