@@ -256,6 +256,14 @@ struct LLLevelArgs {
   int W, H;
 };
 
+// 1 / sigma for the quotient of the u16 remap (div_by), or 0 where the operands
+// may leave its range: the gray of u16 RGB times the scale must keep |g - g_k| at 0
+// or well above the subnormals.
+inline float ll_rsigma(float sigma, float gray_scale) {
+  const bool ok = sigma >= 0x1p-20f && sigma <= 0x1p20f && gray_scale >= 0x1p-30f && gray_scale <= 0x1p-10f;
+  return ok ? 1.0f / sigma : 0.0f;
+}
+
 struct HistArgs {
   ImgView in;               // 1 ch u8
   unsigned int* hist;       // 256 counters

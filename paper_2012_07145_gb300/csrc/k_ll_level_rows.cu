@@ -44,6 +44,7 @@ constexpr int kMaxWarps = 8;             // 256 threads
 struct LevelRowsParams {
   LLLevelArgs a;
   float gk[kK];   // level values k / (K-1), correctly rounded
+  float rsigma;   // level 0: 1 / sigma, correctly rounded (0: divide)
   int strips, rows, units;
   int vec_in;     // level 0: u16 pair loads and stores aligned
   int vec_out;    // pair stores of the output aligned
@@ -53,7 +54,7 @@ struct LevelRowsParams {
 // One fine row of the level-0 input (RGB u16) at the lane's two fine columns.
 struct RGBPair {
   unsigned w[3];
-  __device__ __forceinline__ float get(int c, int j) const { return (float)(j ? (w[c] >> 16) : (w[c] & 0xffffu)); }
+  __device__ __forceinline__ float get(int c, int j) const { return u16_to_f32(w[c], j); }
 };
 
 template <bool LEVEL0, int ODT>
@@ -149,8 +150,13 @@ struct LevelRun {
       }
       ll_interp_index(gK, kK, &k0, &f);
       if (LEVEL0) {
-        g0 = op_ll_remap(gray[j], gks[k0], a.sigma, a.alpha, a.beta);
-        g1 = op_ll_remap(gray[j], gks[k0 + 1], a.sigma, a.alpha, a.beta);
+        if (P.rsigma != 0.0f) {
+          g0 = op_ll_remap_u16(gray[j], gks[k0], a.sigma, P.rsigma, a.alpha, a.beta);
+          g1 = op_ll_remap_u16(gray[j], gks[k0 + 1], a.sigma, P.rsigma, a.alpha, a.beta);
+        } else {
+          g0 = op_ll_remap(gray[j], gks[k0], a.sigma, a.alpha, a.beta);
+          g1 = op_ll_remap(gray[j], gks[k0 + 1], a.sigma, a.alpha, a.beta);
+        }
       } else {
         const float* q = reinterpret_cast<const float*>((const char*)a.G.data + (long long)Y * a.G.rs) + (j ? X1 : X0);
         g0 = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(q) + (long long)k0 * a.G.ps));
@@ -181,15 +187,19 @@ struct LevelRun {
       for (int c = 0; c < 3; ++c) {
         float v[2];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) v[j] = round_storage(ODT, op_ll_colour(rgbf[j][c], gray[j], res[j], a.s_in, a.s_out));
+        for (int j = 0; j < 2; ++j) {
+          v[j] = op_ll_colour(rgbf[j][c], gray[j], res[j], a.s_in, a.s_out);
+          if (ODT != HP_U16) v[j] = round_storage(ODT, v[j]);
+        }
         char* q = row + c * o.ps;
         if (ODT == HP_U16) {
           unsigned short* s = reinterpret_cast<unsigned short*>(q);
+          const unsigned u = f32x2_to_u16x2(v[0], v[1]);
           if (ok1 && P.vec_out) {
-            reinterpret_cast<unsigned*>(s)[X0 >> 1] = (unsigned)(unsigned short)v[0] | ((unsigned)(unsigned short)v[1] << 16);
+            reinterpret_cast<unsigned*>(s)[X0 >> 1] = u;
           } else {
-            s[X0] = (unsigned short)v[0];
-            if (ok1) s[X1] = (unsigned short)v[1];
+            s[X0] = (unsigned short)u;
+            if (ok1) s[X1] = (unsigned short)(u >> 16);
           }
         } else {
           float* s = reinterpret_cast<float*>(q);
@@ -320,6 +330,7 @@ int launch_ll_level_rows(const LLLevelArgs& a, int rows, int threads, int grid, 
   // k / (K-1) in IEEE single precision: the correctly rounded quotient, equal
   // to the device's __fdiv_rn of the same operands.
   for (int k = 0; k < kK; ++k) kp.gk[k] = (float)k / (float)(kK - 1);
+  kp.rsigma = a.level0 ? ll_rsigma(a.sigma, a.gray_scale) : 0.0f;
   kp.strips = (a.Gn.w + kStripW - 1) / kStripW;
   kp.rows = rows;
   kp.units = kp.strips * ((a.Gn.h + rows - 1) / rows);

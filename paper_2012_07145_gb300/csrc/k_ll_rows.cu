@@ -19,10 +19,12 @@
 //
 // Remap cost: outside the band |g - g_k| <= sigma the remap is one
 // multiply-add (op_ll_remap_outside, bit-identical to op_ll_remap there).  The
-// host selects the remap kernel only when no gray value can lie in the band of
-// three levels (sigma below the level spacing 1/(K-1), with a margin for the
-// rounding of g - g_k and of g_k), so the full remap (divide and power) runs
-// for the first two levels of the band at most, whatever the image.
+// host selects the remap kernel only when sigma is below the level spacing
+// 1/(K-1) (with a margin for the rounding of g - g_k, of g_k and of 7 g), so only
+// the levels k0 = floor(7 g) and k0 + 1 can hold g in their bands: the full remap
+// (divide and power) runs for those two, and the other levels take the outside
+// expression, two levels at a time in the paired FP32 instructions, as are the x
+// and y passes.  Bound by issue; 2560x1536 u16: see the kernel.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -41,6 +43,7 @@ constexpr int kStripW = 30;      // coarse columns per warp
 struct LLRowsParams {
   LLDownArgs a;
   float gk[kK];                  // level values k / (K-1), correctly rounded
+  float rsigma;                  // 1 / sigma, correctly rounded (0: divide)
   int strips, rows, units, vec;  // vec: pair loads are aligned (data, row and plane strides)
 };
 
@@ -114,7 +117,7 @@ struct Px;
 template <>
 struct Px<HP_U16> {
   unsigned w[3];
-  __device__ __forceinline__ float get(int c, int j) const { return (float)(j ? (w[c] >> 16) : (w[c] & 0xffffu)); }
+  __device__ __forceinline__ float get(int c, int j) const { return u16_to_f32(w[c], j); }
   __device__ __forceinline__ void load(const char* row, long long ps, int cx0, int cx1, bool pair) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -147,6 +150,62 @@ struct Px<HP_F32> {
   }
 };
 
+typedef unsigned long long u64;
+
+__device__ __forceinline__ u64 pack2(float a, float b) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(u64 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+  u64 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+  u64 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ u64 dup2(float a) { return pack2(a, a); }
+
+// xpass() of two channels at once (the same operations per channel).
+__device__ __forceinline__ u64 xpass2(u64 v0, u64 v1) {
+  float a0, a1, b0, b1;
+  unpack2(v0, a0, a1);
+  unpack2(v1, b0, b1);
+  const u64 l0 = pack2(__shfl_up_sync(0xffffffffu, a0, 1), __shfl_up_sync(0xffffffffu, a1, 1));
+  const u64 l1 = pack2(__shfl_up_sync(0xffffffffu, b0, 1), __shfl_up_sync(0xffffffffu, b1, 1));
+  const u64 r0 = pack2(__shfl_down_sync(0xffffffffu, a0, 1), __shfl_down_sync(0xffffffffu, a1, 1));
+  u64 s = mul2(dup2(0.0625f), l0);
+  s = fma2(dup2(0.25f), l1, s);
+  s = fma2(dup2(0.375f), v0, s);
+  s = fma2(dup2(0.25f), v1, s);
+  return fma2(dup2(0.0625f), r0, s);
+}
+
+// ytaps() of two channels at once.
+template <int PH>
+__device__ __forceinline__ u64 ytaps2(u64 (&acc)[3], u64 h) {
+  constexpr int m = PH >> 1;
+  u64 fin = 0;
+  if ((PH & 1) == 0) {
+    fin = fma2(dup2(0.0625f), h, acc[(m + 1) % 3]);
+    acc[(m + 2) % 3] = fma2(dup2(0.375f), h, acc[(m + 2) % 3]);
+    acc[m] = mul2(dup2(0.0625f), h);
+  } else {
+    acc[m] = fma2(dup2(0.25f), h, acc[m]);
+    acc[(m + 2) % 3] = fma2(dup2(0.25f), h, acc[(m + 2) % 3]);
+  }
+  return fin;
+}
+
 // The remap source: gray of the input, its K remaps and gray itself.
 // F32S: gray, remap and output stored as f32 (no rounding steps).
 template <int IDT, bool F32S>
@@ -154,7 +213,8 @@ struct RemapRun {
   const LLRowsParams& P;
   const float* gks;    // the level table in shared memory (dynamic index)
   RunGeom G;
-  float acc[kC][3];
+  u64 acc[kK / 2][3];  // levels 2 p and 2 p + 1
+  float acc_g[3];      // gray
   Px<IDT> cur, nxt;
 
   __device__ __forceinline__ RemapRun(const LLRowsParams& p, const float* g) : P(p), gks(g) {}
@@ -174,53 +234,73 @@ struct RemapRun {
     }
   }
 
+  __device__ __forceinline__ float remap(float g, float gk) const {
+    const LLDownArgs& a = P.a;
+    if (IDT == HP_U16 && F32S && P.rsigma != 0.0f) return op_ll_remap_u16(g, gk, a.sigma, P.rsigma, a.alpha, a.beta);
+    return op_ll_remap(g, gk, a.sigma, a.alpha, a.beta);
+  }
+
+  // The remap outside the band for levels 2 p and 2 p + 1 (op_ll_remap_outside's operations).
+  __device__ __forceinline__ u64 outside2(float g, int p) const {
+    const LLDownArgs& a = P.a;
+    const u64 gk = pack2(P.gk[2 * p], P.gk[2 * p + 1]);
+    const u64 d = fma2(gk, dup2(-1.0f), dup2(g));   // g - g_k, one rounding
+    float d0, d1, m0, m1;
+    unpack2(d, d0, d1);
+    const u64 m = fma2(dup2(a.beta), add2(pack2(fabsf(d0), fabsf(d1)), dup2(-a.sigma)), dup2(a.sigma));
+    unpack2(m, m0, m1);
+    return add2(gk, pack2(copysignf(m0, d0), copysignf(m1, d1)));
+  }
+
   template <int PH>
   __device__ __forceinline__ void row(int t) {
     const LLDownArgs& a = P.a;
     if (t + 1 < G.T) fetch(nxt, t + 1);
     float g[2], pa[2], pb[2];
-    int ka[2], kb[2];
+    int k0[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       g[j] = rs(a.st_gray, op_gray(cur.get(0, j), cur.get(1, j), cur.get(2, j), a.gray_scale));
-      unsigned m = 0;
-#pragma unroll
-      for (int k = 0; k < kK; ++k) m |= fabsf(__fsub_rn(g[j], P.gk[k])) <= a.sigma ? 1u << k : 0u;
-      ka[j] = __ffs(m) - 1;            // first level in the band, -1 if none
-      kb[j] = __ffs(m & (m - 1)) - 1;  // second level, -1 if none
-      pa[j] = op_ll_remap(g[j], gks[ka[j] & (kK - 1)], a.sigma, a.alpha, a.beta);
-      pb[j] = op_ll_remap(g[j], gks[kb[j] & (kK - 1)], a.sigma, a.alpha, a.beta);
+      k0[j] = iclamp(__float2int_rd(__fmul_rn(g[j], (float)(kK - 1))), 0, kK - 2);
+      pa[j] = remap(g[j], gks[k0[j]]);
+      pb[j] = remap(g[j], gks[k0[j] + 1]);
     }
     const int ofin = (t >> 1) - 2;
     const bool st = (PH & 1) == 0 && G.prod && ofin >= 0 && ofin < G.nout;
 #pragma unroll
-    for (int c = 0; c < kC; ++c) {
-      float v[2];
+    for (int p = 0; p < kK / 2; ++p) {
+      u64 v[2];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        float r;
-        if (c < kK) {
-          const float d = __fsub_rn(g[j], P.gk[c]);
-          r = op_ll_remap_outside(d, fabsf(d), P.gk[c], a.sigma, a.beta);
-          r = c == ka[j] ? pa[j] : r;
-          r = c == kb[j] ? pb[j] : r;
-        } else {
-          r = g[j];
-        }
-        v[j] = rs(a.st_remap, r);
+        float r0, r1;
+        unpack2(outside2(g[j], p), r0, r1);
+        r0 = k0[j] == 2 * p ? pa[j] : r0;
+        r0 = k0[j] == 2 * p - 1 ? pb[j] : r0;
+        r1 = k0[j] == 2 * p + 1 ? pa[j] : r1;
+        r1 = k0[j] == 2 * p ? pb[j] : r1;
+        v[j] = pack2(rs(a.st_remap, r0), rs(a.st_remap, r1));
       }
-      const float fin = ytaps<PH>(acc[c], xpass(v[0], v[1]));
-      if (st) store(c, G.y0 + ofin, fin);
+      const u64 fin = ytaps2<PH>(acc[p], xpass2(v[0], v[1]));
+      if (st) {
+        float f0, f1;
+        unpack2(fin, f0, f1);
+        store(2 * p, G.y0 + ofin, f0);
+        store(2 * p + 1, G.y0 + ofin, f1);
+      }
     }
+    const float fin = ytaps<PH>(acc_g, xpass(rs(a.st_remap, g[0]), rs(a.st_remap, g[1])));
+    if (st) store(kK, G.y0 + ofin, fin);
     cur = nxt;
   }
 
   __device__ __forceinline__ void run(int strip, int run_idx) {
     G.init(strip, run_idx, P.rows, P.a.src.w, P.a.out.w, P.a.out.h, P.vec);
 #pragma unroll
-    for (int c = 0; c < kC; ++c)
+    for (int s = 0; s < 3; ++s) {
+      acc_g[s] = 0.0f;
 #pragma unroll
-      for (int s = 0; s < 3; ++s) acc[c][s] = 0.0f;
+      for (int p = 0; p < kK / 2; ++p) acc[p][s] = 0;
+    }
     fetch(cur, 0);
     walk_rows(*this, G.T);
   }
@@ -413,6 +493,7 @@ int launch_ll_remap_rows(const LLDownArgs& a, int rows, int threads, int grid, v
   // k / (K-1) in IEEE single precision: the correctly rounded quotient, equal
   // to the device's __fdiv_rn of the same operands.
   for (int k = 0; k < kK; ++k) kp.gk[k] = (float)k / (float)(kK - 1);
+  kp.rsigma = ll_rsigma(a.sigma, a.gray_scale);
   kp.strips = (a.out.w + kStripW - 1) / kStripW;
   kp.rows = rows;
   kp.units = kp.strips * ((a.out.h + rows - 1) / rows);

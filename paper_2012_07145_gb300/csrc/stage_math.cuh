@@ -135,6 +135,42 @@ __device__ __forceinline__ float op_ll_remap(float i, float g, float sigma, floa
   return ad == 0.0f ? g : __fadd_rn(g, copysignf(mag, d));
 }
 
+// a / b, correctly rounded, for 0 <= a < 2^7 with a = 0 or a > 2^-60 and b in
+// [2^-20, 2^20], given rb = 1 / b correctly rounded (Markstein's iteration,
+// 1990: two residual corrections by fused multiply-adds; the first leaves the
+// quotient within an ulp, the second rounds it).  Five FP32 operations.
+__device__ __forceinline__ float div_by(float a, float b, float rb) {
+  float q = __fmul_rn(a, rb);
+  q = __fmaf_rn(__fmaf_rn(-q, b, a), rb, q);
+  return __fmaf_rn(__fmaf_rn(-q, b, a), rb, q);
+}
+
+// op_ll_remap where i is a gray of u16 RGB (|i - g| is 0 or above 2^-60), given
+// rsigma = 1 / sigma correctly rounded.
+__device__ __forceinline__ float op_ll_remap_u16(float i, float g, float sigma, float rsigma, float alpha, float beta) {
+  const float d = __fsub_rn(i, g);
+  const float ad = fabsf(d);
+  const float x = div_by(ad, sigma, rsigma);
+  const float inside = __fmul_rn(sigma, __powf(x, alpha));
+  const float outside = __fmaf_rn(beta, __fsub_rn(ad, sigma), sigma);
+  const float mag = ad <= sigma ? inside : outside;
+  return ad == 0.0f ? g : __fadd_rn(g, copysignf(mag, d));
+}
+
+// The low (hi = 0) or high u16 of w as a float: 2^23 + u is exact in f32, so one
+// byte permutation and one subtraction stand for the conversion.
+__device__ __forceinline__ float u16_to_f32(unsigned w, int hi) {
+  return __fsub_rn(__uint_as_float(__byte_perm(w, 0x4b000000u, hi ? 0x7432 : 0x7410)), 8388608.0f);
+}
+
+// clamp(rint(a), 0, 65535) of two values, packed: adding 2^23 rounds to an
+// integer (half to even) in the low bits.
+__device__ __forceinline__ unsigned f32x2_to_u16x2(float a, float b) {
+  const float x = __fadd_rn(fminf(fmaxf(a, 0.0f), 65535.0f), 8388608.0f);
+  const float y = __fadd_rn(fminf(fmaxf(b, 0.0f), 65535.0f), 8388608.0f);
+  return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x5410);
+}
+
 // The remap outside the band (|d| > sigma), bit-identical to op_ll_remap there.
 __device__ __forceinline__ float op_ll_remap_outside(float d, float ad, float g, float sigma, float beta) {
   return __fadd_rn(g, copysignf(__fmaf_rn(beta, __fsub_rn(ad, sigma), sigma), d));
