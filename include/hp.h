@@ -325,6 +325,8 @@ hp_status hp_infer_bounds(hp_pipeline* p, const int* in_widths, const int* in_he
  *   it with one cudaGraphLaunch on the caller's stream.  Up to 16 graphs are
  *   kept per input size (least recently used evicted).  Capture happens on a
  *   private stream, so the caller's stream may be the legacy default stream.
+ *   A realize that is one kernel of at least 9728 threads is launched directly
+ *   all the same: it then starts as the previous kernel on the stream drains.
  * HP_OPT_OVERLAP (0/1, default 1): launch the kernels of a realize with
  *   programmatic dependent launch, so that a kernel's blocks may be scheduled
  *   while its predecessor's last blocks drain.  Every kernel waits for its

@@ -248,8 +248,11 @@ class Pipeline:
 
     def realize(self, inputs, output, stream=None):
         """inputs: list of Buffer (device); output: Buffer (device); stream: cudaStream_t as int or None."""
-        arr = (Buffer * len(inputs))(*inputs)
-        check(lib().hp_realize(self.h, arr, len(inputs), ctypes.byref(output), ctypes.c_void_p(stream or 0)))
+        n = len(inputs)
+        arr = ctypes.byref(inputs[0]) if n == 1 else (Buffer * n)(*inputs)   # one buffer is its own array
+        st = _lib.hp_realize(self.h, arr, n, ctypes.byref(output), stream)
+        if st != HP_OK:
+            check(st)
 
     def prepare(self, sizes, stream=None):
         """Lowers and allocates for inputs of the given (w, h) sizes without running."""
