@@ -184,9 +184,10 @@ struct GridArgs {
 };
 
 // Pair layout of a blurred grid that only slices read: [gy][gx][level][2], value
-// and weight of a level together; a cell's levels padded to an even number, so
-// two levels are one aligned 128-bit store.
-HPHD int grid_pair_levels(int gz) { return (gz + 1) & ~1; }
+// and weight of a level together; the last level twice (a slice reads a level and
+// the next), and an even number of levels per cell, so that two levels are one
+// aligned 128-bit store.
+HPHD int grid_pair_levels(int gz) { return (gz + 2) & ~1; }
 
 // Blur of a bilateral grid (k_grid.cu): [1,4,6,4,1]/16 along the range levels,
 // then x, then y; rows per run of the streaming kernel.

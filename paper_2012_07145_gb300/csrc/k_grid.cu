@@ -192,14 +192,15 @@ __device__ __forceinline__ u64 lerp2(u64 a, u64 b, float f) {
 }
 
 // The slice of a grid in pair layout (see grid_pair_levels): a cell's (value,
-// weight) pairs lie together, level by level, so a corner of a pixel's two range
-// levels is two adjacent 64-bit loads instead of four 32-bit ones from four
-// planes, and the pair is interpolated by the paired FP32 instructions.  A warp
-// takes 32 consecutive pixels of 4 rows: at s = 8 a load of the warp touches the
-// levels of 4 cells (a few cache lines), where four pixels of a row per thread
-// touched 16.  SAME: the cell size is a power of two >= 4, so a thread's four
-// pixels (rows 4 q .. 4 q + 3 of a column) lie in one cell.
-template <bool SAME>
+// weight) pairs lie together, level by level, the last level twice, so a corner of
+// a pixel's two range levels is two adjacent 64-bit loads at one address instead
+// of four 32-bit ones from four planes, and the pair is interpolated by the paired
+// FP32 instructions.  Bound by issue: 2560x1536, s = 8, 11 levels: 28.2 us from
+// planes, 18.8 as pairs with clamped levels and a type switch per pixel, about 14
+// so.  SAME: the cell size is a power of two >= 4,
+// so a thread's four pixels (rows 4 q .. 4 q + 3 of a column) lie in one cell, whose
+// corner addresses they share.  F32: the image is f32.
+template <bool SAME, bool F32>
 __global__ void __launch_bounds__(256) k_grid_slice_pairs(const GridArgs a) {
   grid_dep_sync();
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
@@ -209,31 +210,43 @@ __global__ void __launch_bounds__(256) k_grid_slice_pairs(const GridArgs a) {
   const int gw = a.grid.w, gh = a.grid.h, gzp = grid_pair_levels(a.gz);
   const float gxf = __fmul_rn((float)x, a.inv_s);
   const float flx = floorf(gxf), fx = __fsub_rn(gxf, flx);
-  const u64* const c0 = (const u64*)a.grid.data + (long long)iclamp((int)flx, 0, gw - 1) * gzp;
-  const u64* const c1 = (const u64*)a.grid.data + (long long)iclamp((int)flx + 1, 0, gw - 1) * gzp;
-  const int pitch = gw * gzp;   // pairs per grid row
+  const int x0 = iclamp((int)flx, 0, gw - 1) * gzp, x1 = iclamp((int)flx + 1, 0, gw - 1) * gzp;
+  const u64* const g = (const u64*)a.grid.data;
+  const long long pitch = (long long)gw * gzp;   // pairs per grid row
+  const u64 *b00 = g, *b10 = g, *b01 = g, *b11 = g;   // the cell's corners at level 0
   float v[4];
+  {
+    const char* p = (const char*)a.in.data + (long long)yb * a.in.rs;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = gray_at(a.in, x, imin(yb + k, H - 1));
-  int r0 = 0, r1 = 0;
+    for (int k = 0; k < 4; ++k) {
+      const float t = F32 ? __ldg(reinterpret_cast<const float*>(p) + x) : load_px(a.in, 0, x, imin(yb + k, H - 1));
+      v[k] = fminf(fmaxf(t, 0.0f), 1.0f);
+      if (yb + k + 1 < H) p += a.in.rs;
+    }
+  }
+  float fly = 0.0f;
+  char* q = (char*)a.out.data + (long long)yb * a.out.rs + 4LL * x;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const float gyf = __fmul_rn((float)(yb + k), a.inv_s), gzf = __fmul_rn(v[k], a.inv_r);
-    const float fly = floorf(gyf), flz = floorf(gzf);
-    const float fy = __fsub_rn(gyf, fly), fz = __fsub_rn(gzf, flz);
     if (!SAME || k == 0) {
-      r0 = iclamp((int)fly, 0, gh - 1) * pitch;
-      r1 = iclamp((int)fly + 1, 0, gh - 1) * pitch;
+      fly = floorf(gyf);
+      const u64* r0 = g + iclamp((int)fly, 0, gh - 1) * pitch;
+      const u64* r1 = g + iclamp((int)fly + 1, 0, gh - 1) * pitch;
+      b00 = r0 + x0; b10 = r0 + x1; b01 = r1 + x0; b11 = r1 + x1;
     }
-    const int z0 = iclamp((int)flz, 0, a.gz - 1), z1 = iclamp((int)flz + 1, 0, a.gz - 1);
-    const u64 lo = lerp2(lerp2(__ldg(c0 + r0 + z0), __ldg(c1 + r0 + z0), fx),
-                         lerp2(__ldg(c0 + r1 + z0), __ldg(c1 + r1 + z0), fx), fy);
-    const u64 hi = lerp2(lerp2(__ldg(c0 + r0 + z1), __ldg(c1 + r0 + z1), fx),
-                         lerp2(__ldg(c0 + r1 + z1), __ldg(c1 + r1 + z1), fx), fy);
+    // 0 <= v <= 1, so the level is in [0, gz - 1] without a clamp and the next
+    // one is in the layout
+    const int z = (int)gzf;
+    const float fy = __fsub_rn(gyf, fly), fz = __fsub_rn(gzf, (float)z);
+    const u64 lo = lerp2(lerp2(__ldg(b00 + z), __ldg(b10 + z), fx), lerp2(__ldg(b01 + z), __ldg(b11 + z), fx), fy);
+    const u64 hi = lerp2(lerp2(__ldg(b00 + z + 1), __ldg(b10 + z + 1), fx),
+                         lerp2(__ldg(b01 + z + 1), __ldg(b11 + z + 1), fx), fy);
     float val, wt;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(val), "=f"(wt) : "l"(lerp2(lo, hi, fz)));
     const float o = wt > 0.0f ? __fdiv_rn(val, wt) : v[k];
-    if (yb + k < H) reinterpret_cast<float*>((char*)a.out.data + (long long)(yb + k) * a.out.rs)[x] = o;
+    if (yb + k < H) *reinterpret_cast<float*>(q) = o;
+    q += a.out.rs;
   }
 }
 
@@ -258,7 +271,8 @@ int launch_grid_slice(const GridArgs& a, void* stream) {
   if (a.gz < 1 || a.grid.dtype != HP_F32 || a.out.dtype != HP_F32 || a.grid.c < 2 * a.gz) return (int)cudaErrorInvalidValue;
   dim3 grid((a.in.w + 127) / 128, (a.in.h + 7) / 8, 1);
   if (a.pairs) grid = dim3((a.in.w + 31) / 32, (a.in.h + 31) / 32, 1);
-  auto kern = !a.pairs ? k_grid_slice : a.s >= 4 && (a.s & (a.s - 1)) == 0 ? k_grid_slice_pairs<true> : k_grid_slice_pairs<false>;
+  auto kern = !a.pairs ? k_grid_slice : a.in.dtype != HP_F32 ? k_grid_slice_pairs<false, false>
+              : a.s >= 4 && (a.s & (a.s - 1)) == 0 ? k_grid_slice_pairs<true, true> : k_grid_slice_pairs<false, true>;
   { const int le_ = launch_kernel(kern, grid, dim3(256), 0, stream, a); if (le_) return le_; }
   __atomic_add_fetch(&g_launches, 1ULL, __ATOMIC_RELAXED);
   return (int)cudaGetLastError();
@@ -342,10 +356,15 @@ struct BlurRun {
     if (P.a.pairs) {
       const int gzp = grid_pair_levels(P.a.gz);
       float* p = (float*)o.data + (((long long)(y0 + ofin) * o.w + x) * gzp + z0) * 2;
+      // level gz holds level gz - 1 again
+#pragma unroll
+      for (int q = kZC - 1; q > 0; --q)
+        if (z0 + q == P.a.gz) { done[0][q] = done[0][q - 1]; done[1][q] = done[1][q - 1]; }
 #pragma unroll
       for (int q = 0; q < kZC; q += 2)
         if (z0 + q < gzp)
           *reinterpret_cast<float4*>(p + 2 * q) = make_float4(done[0][q], done[1][q], done[0][q + 1], done[1][q + 1]);
+      if (z0 + kZC == P.a.gz) *reinterpret_cast<float2*>(p + 2 * kZC) = make_float2(done[0][kZC - 1], done[1][kZC - 1]);
     } else {
 #pragma unroll
       for (int q = 0; q < kZC; ++q)
