@@ -257,6 +257,19 @@ struct LLLevelArgs {
   int W, H;
 };
 
+// The coarse end of an interpolate or local-Laplacian pyramid (k_pyr_tail.cu):
+// level 0 of the tail is read, its result (I or R) written.
+constexpr int kTailLevels = 16;
+constexpr int kTailPixels = 1024;   // of the tail's finest level: larger ones keep one CTA busy for longer than their
+                                    // launches take (interpolate 2559x1535, 10 levels: 103.0 us without a tail, 98.6 at
+                                    // 1024, 104.4 at 4096; 400x300, 8 levels: 35.5, 30.7, 33.1)
+struct PyrTailArgs {
+  ImgView src, out;
+  int levels, channels;    // channels of a level's stack
+  int ll, K, rn_ch;        // local Laplacian: levels K, channel of the coarsest stack that is its result
+  int w[kTailLevels], h[kTailLevels];
+};
+
 // 1 / sigma for the quotient of the u16 remap (div_by), or 0 where the operands
 // may leave its range: the gray of u16 RGB times the scale must keep |g - g_k| at 0
 // or well above the subnormals.
@@ -350,6 +363,8 @@ int interp_rows_grid(const InterpArgs& a, int units, int threads);
 // dynamic shared memory of the interpolate level kernel (the per-warp TMA rings of the fine level)
 int interp_rows_smem_bytes(int threads);
 int launch_interp_rows(const InterpArgs& a, int grid, void* stream);
+int pyr_tail_smem_bytes(const PyrTailArgs& a);
+int launch_pyr_tail(const PyrTailArgs& a, void* stream);
 int pw_rows_op_ok(int op);
 int launch_pw_rows(const PwArgs& p, void* stream);
 int grid_max_levels();

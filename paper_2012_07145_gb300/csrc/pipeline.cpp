@@ -107,7 +107,10 @@ struct GroupPlan {
   LLRoles llroles{};
   std::unique_ptr<GPlan> gplan;
   bool rows_given = false;    // the schedule sets the rows per run
-  bool folded = false;        // computed inside its consumers: no launch, no buffer
+  bool folded = false;        // computed inside its consumers or a pyramid tail: no launch, no buffer
+  bool tail = false;          // the group's launch is a pyramid tail, from tail_src
+  int tail_src = 0;
+  PyrTailArgs tail_args{};
   std::vector<int> ext_refs;  // generic: external refs (stage id or -1-k)
   size_t aux_bytes = 0;       // kernel state kept across launches (zeroed once at allocation)
   void* aux = nullptr;
@@ -1296,6 +1299,98 @@ hp_status plan_premul_fold(hp_pipeline* p, Plan& plan) {
   return HP_OK;
 }
 
+// Whether only the given groups read a stage (and it is not the output).
+bool read_only_by(const hp_pipeline* p, const Plan& plan, int ref, const std::vector<const GroupPlan*>& by) {
+  if (ref < 0 || ref == p->output) return false;
+  for (const GroupPlan& g : plan.groups) {
+    if (std::find(by.begin(), by.end(), &g) != by.end()) continue;
+    for (int s : g.members)
+      for (int r : p->stages[s].inputs)
+        if (r == ref) return false;
+  }
+  return true;
+}
+
+// The coarse end of a pyramid as one launch: walks up from the coarsest level
+// step (its coarse image is a downsample of its fine one) through steps whose
+// coarse result is the step below's output, as long as the level fits a tail and
+// everything inside is read inside alone.  The last step taken launches the tail;
+// the other steps and the downsamples between are folded into it.  Worth it from
+// two steps (four launches) on.
+void plan_pyr_tail(const hp_pipeline* p, Plan& plan) {
+  auto maker = [&](int ref, int kernel) -> GroupPlan* {
+    for (GroupPlan& g : plan.groups)
+      if (!g.folded && g.output == ref && g.kernel == kernel) return &g;
+    return nullptr;
+  };
+  for (const bool ll : {false, true}) {
+    const int kernel = ll ? HP_KERNEL_LL_LEVEL_ROWS : HP_KERNEL_INTERP_ROWS;
+    auto usable = [&](const GroupPlan& g) {
+      return g.kernel == kernel && !g.folded && !g.tail && !(ll ? g.lllevel.level0 : g.interp.final_div || g.interp.premul);
+    };
+    auto fine_of = [&](const GroupPlan& g) { return ll ? g.llroles.Gl : g.ext_refs[0]; };
+    auto stack_of = [&](const GroupPlan& g) { return ll ? g.llroles.Gn : g.ext_refs[1]; };  // interpolate: I_{l+1}
+    for (GroupPlan& start : plan.groups) {
+      if (!usable(start)) continue;
+      // the coarsest step: its coarse image is the coarsest level itself
+      if (ll && (start.llroles.select < 0 || p->stages[start.llroles.select].inputs[0] != start.llroles.Gn)) continue;
+      GroupPlan* down = maker(stack_of(start), HP_KERNEL_LL_DOWN_ROWS);
+      if (!down || down->ext_refs[0] != fine_of(start) || down->lldown.premul) continue;
+      PyrTailArgs t{};
+      t.ll = ll;
+      t.channels = stage_channels_of_ref(p, fine_of(start));
+      t.K = ll ? start.lllevel.K : 0;
+      t.rn_ch = ll ? start.lllevel.rn_ch : 0;
+      if (ll ? t.channels != t.K + 1 : t.channels != 4) continue;
+      std::vector<const GroupPlan*> in = {&start, down};   // steps and downsamples, coarsest first
+      std::vector<GroupPlan*> all = {down, &start};
+      std::vector<int> refs = {stack_of(start), fine_of(start)};  // the level stacks, coarsest first
+      auto fits = [&](const std::vector<int>& r) {
+        if ((int)r.size() > kTailLevels) return false;
+        PyrTailArgs q = t;
+        q.levels = (int)r.size();
+        for (int l = 0; l < q.levels; ++l) {
+          const Dom d = dom_of_ref(plan, r[q.levels - 1 - l]);
+          q.w[l] = d.w;
+          q.h[l] = d.h;
+        }
+        if (!pyr_tail_smem_bytes(q)) return false;
+        t = q;
+        return true;
+      };
+      if (!read_only_by(p, plan, stack_of(start), in) || !fits(refs)) continue;
+      GroupPlan* last = &start;
+      while (true) {
+        GroupPlan* next = nullptr;
+        for (GroupPlan& g : plan.groups)
+          if (usable(g) && (ll ? g.llroles.select < 0 && g.llroles.Rn == last->output && g.llroles.Gn == fine_of(*last)
+                               : g.ext_refs[1] == last->output))
+            next = &g;
+        GroupPlan* d = next ? maker(fine_of(*last), HP_KERNEL_LL_DOWN_ROWS) : nullptr;
+        if (!next || !d || d->ext_refs[0] != fine_of(*next) || d->lldown.premul ||
+            stage_channels_of_ref(p, fine_of(*next)) != t.channels)
+          break;
+        std::vector<const GroupPlan*> in2 = in;
+        in2.push_back(next);
+        in2.push_back(d);
+        std::vector<int> refs2 = refs;
+        refs2.push_back(fine_of(*next));
+        if (!read_only_by(p, plan, last->output, in2) || !read_only_by(p, plan, fine_of(*last), in2) || !fits(refs2)) break;
+        in = in2;
+        refs = refs2;
+        all.push_back(d);
+        all.push_back(next);
+        last = next;
+      }
+      if (t.levels < 3) continue;
+      for (GroupPlan* g : all) g->folded = g != last;
+      last->tail = true;
+      last->tail_src = refs.back();
+      last->tail_args = t;
+    }
+  }
+}
+
 // A blurred grid that nothing but slices reads goes to them in pair layout.
 void plan_grid_pairs(const hp_pipeline* p, Plan& plan) {
   for (GroupPlan& b : plan.groups) {
@@ -1590,7 +1685,9 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
                                       "(fused Harris or histogram equalization)", p->batch);
   }
   plan_grid_pairs(p, plan);
-  return plan_premul_fold(p, plan);
+  if ((s = plan_premul_fold(p, plan))) return s;
+  plan_pyr_tail(p, plan);
+  return HP_OK;
 }
 
 // First realize of a plan: its buffers.  Kernel state is cleared on the
@@ -1724,6 +1821,13 @@ hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, c
     if (gp.folded) continue;
     ImgView out = ref_view(p, plan, gp.output, inputs, output);
     int e = 0;
+    if (gp.tail) {
+      PyrTailArgs a = gp.tail_args;
+      a.src = ref_view(p, plan, gp.tail_src, inputs, output);
+      a.out = out;
+      if ((e = launch_pyr_tail(a, stream))) return cuda_fail(e, "kernel launch");
+      continue;
+    }
     switch (gp.kernel) {
       case HP_KERNEL_STENCIL_CHAIN:
       case HP_KERNEL_UNSHARP:
