@@ -71,7 +71,7 @@ struct LevelRun {
 
   __device__ __forceinline__ LevelRun(const LevelRowsParams& p, const float* g, float* w) : P(p), gks(g), win(w) {}
 
-  __device__ __forceinline__ void load_raw(int q) {
+  __device__ __forceinline__ void load_raw(int q, float (&raw)[kNC]) const {
     const LLLevelArgs& a = P.a;
     const int cy = iclamp(n0 - 1 + q, 0, a.Gn.h - 1);
     const char* g = (const char*)a.Gn.data + (long long)cy * a.Gn.rs;
@@ -82,9 +82,9 @@ struct LevelRun {
                                                    (long long)ry * a.Rn.rs) + iclamp(m, 0, a.Rn.w - 1));
   }
 
-  // x pass of the loaded coarse row into window slot S
+  // x pass of a loaded coarse row into window slot S
   template <int S>
-  __device__ __forceinline__ void xpass() {
+  __device__ __forceinline__ void xpass(const float (&raw)[kNC]) {
 #pragma unroll
     for (int c = 0; c < kNC; ++c) {
       const float l = __shfl_up_sync(0xffffffffu, raw[c], 1);
@@ -227,8 +227,8 @@ struct LevelRun {
   template <int PH>
   __device__ __forceinline__ void step(int i) {
     constexpr int A = PH, B = (PH + 1) % 3, C = (PH + 2) % 3;
-    xpass<C>();
-    if (i + 3 <= nrun + 1) load_raw(i + 3);
+    xpass<C>(raw);
+    if (i + 3 <= nrun + 1) load_raw(i + 3, raw);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       pin[r] = pin_nxt[r];
@@ -252,12 +252,25 @@ struct LevelRun {
     ok1 = prod && 2 * m + 1 <= a.W - 1;
     n0 = run_idx * P.rows;
     nrun = imin(P.rows, a.Gn.h - n0);  // coarse rows n0 .. n0+nrun-1 give fine rows 2n, 2n+1
-    load_raw(0);
-    xpass<0>();
-    load_raw(1);
-    xpass<1>();
-    load_raw(2);
-    load_step(0, pin_nxt, gkp_nxt);
+    if (LEVEL0) {
+      load_raw(0, raw);
+      xpass<0>(raw);
+      load_raw(1, raw);
+      xpass<1>(raw);
+      load_raw(2, raw);
+      load_step(0, pin_nxt, gkp_nxt);
+    } else {
+      // the run's first loads all in flight: a coarse level is a few rows per
+      // run, and each wait for memory is as long as the rest of a row (level 0
+      // has longer runs and no registers to spare)
+      float r0[kNC], r1[kNC];
+      load_raw(0, r0);
+      load_raw(1, r1);
+      load_raw(2, raw);
+      load_step(0, pin_nxt, gkp_nxt);
+      xpass<0>(r0);
+      xpass<1>(r1);
+    }
     for (int i = 0; i < nrun; i += 3) {
       step<0>(i);
       if (i + 1 >= nrun) break;

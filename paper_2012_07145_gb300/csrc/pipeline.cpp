@@ -1163,8 +1163,9 @@ hp_status build_ll_rows(const hp_pipeline* p, const Plan& plan, GroupPlan& gp) {
   };
   if (gp.tile_h == 0) {
     const long long warps = (long long)grid_for(1 << 30) * (gp.threads / 32);
-    gp.tile_h = remap ? default_run_rows(od.h, units_per_row, warps)
-                      : (int)std::max(1LL, ((long long)od.h * units_per_row + warps - 1) / warps);
+    // on a small image short runs, although half of what they read is warm-up:
+    // the rows of a run are one wait for memory each
+    gp.tile_h = (int)std::max(remap ? 2LL : 1LL, ((long long)od.h * units_per_row + warps - 1) / warps);
   }
   if (gp.tile_h < 1 || gp.tile_h > 65536) return fail(HP_ERR_SCHEDULE, "streaming downsample needs tile_h >= 1");
   a.tile_h = gp.tile_h;
