@@ -67,7 +67,7 @@ struct LevelRun {
   float hr[3][2];        // x-passed coarse rows of R_{l+1} (window slot, fine column)
   float raw[kNC];        // the next coarse row, in flight
   RGBPair pin[2], pin_nxt[2];   // level 0: input rows 2n, 2n+1 of this step and the next
-  float2 gkp[2], gkp_nxt[2];    // above level 0: G_l[K] at rows 2n, 2n+1
+  float2 gkp_nxt[2];            // above level 0: G_l[K] at rows 2n, 2n+1 of the next step
 
   __device__ __forceinline__ LevelRun(const LevelRowsParams& p, const float* g, float* w) : P(p), gks(g), win(w) {}
 
@@ -129,27 +129,38 @@ struct LevelRun {
     load_px_row(imin(Y + 1, P.a.H - 1), rgb[1], gk[1]);
   }
 
+  // Above level 0: the two levels' values that a fine row's pixels blend.
+  struct Gathered {
+    int k0[2];
+    float f[2], lo[2], hi[2];
+  };
+  __device__ __forceinline__ void gather(int Y, float2 gkv, Gathered& t) const {
+    const LLLevelArgs& a = P.a;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      ll_interp_index(j ? gkv.y : gkv.x, kK, &t.k0[j], &t.f[j]);
+      const char* q = (const char*)a.G.data + (long long)Y * a.G.rs + 4LL * (j ? X1 : X0) + (long long)t.k0[j] * a.G.ps;
+      t.lo[j] = __ldg(reinterpret_cast<const float*>(q));
+      t.hi[j] = __ldg(reinterpret_cast<const float*>(q + a.G.ps));
+    }
+  }
+
   // Fine row Y from the window slots of coarse rows n-1 (A), n (B), n+1 (C);
   // odd rows use B and C only.
   template <bool ODD, int A, int B, int C>
-  __device__ __forceinline__ void emit(int Y, const RGBPair& rgb, float2 gkv) const {
+  __device__ __forceinline__ void emit(int Y, const RGBPair& rgb, const Gathered& t) const {
     const LLLevelArgs& a = P.a;
     float res[2], gray[2], rgbf[2][3];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      float gK, g0, g1;
+      float g0, g1;
       int k0;
       float f;
       if (LEVEL0) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) rgbf[j][c] = rgb.get(c, j);
         gray[j] = op_gray(rgbf[j][0], rgbf[j][1], rgbf[j][2], a.gray_scale);
-        gK = gray[j];
-      } else {
-        gK = j ? gkv.y : gkv.x;
-      }
-      ll_interp_index(gK, kK, &k0, &f);
-      if (LEVEL0) {
+        ll_interp_index(gray[j], kK, &k0, &f);
         if (P.rsigma != 0.0f) {
           g0 = op_ll_remap_u16(gray[j], gks[k0], a.sigma, P.rsigma, a.alpha, a.beta);
           g1 = op_ll_remap_u16(gray[j], gks[k0 + 1], a.sigma, P.rsigma, a.alpha, a.beta);
@@ -158,9 +169,10 @@ struct LevelRun {
           g1 = op_ll_remap(gray[j], gks[k0 + 1], a.sigma, a.alpha, a.beta);
         }
       } else {
-        const float* q = reinterpret_cast<const float*>((const char*)a.G.data + (long long)Y * a.G.rs) + (j ? X1 : X0);
-        g0 = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(q) + (long long)k0 * a.G.ps));
-        g1 = __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(q) + (long long)(k0 + 1) * a.G.ps));
+        k0 = t.k0[j];
+        f = t.f[j];
+        g0 = t.lo[j];
+        g1 = t.hi[j];
       }
       // y pass of the two levels this pixel blends (k0 and k0 + 1), and of R
       const float* wl = win + (2 * k0 + j) * 32;  // level k0, this column; level k0 + 1 is 64 further
@@ -227,17 +239,19 @@ struct LevelRun {
   template <int PH>
   __device__ __forceinline__ void step(int i) {
     constexpr int A = PH, B = (PH + 1) % 3, C = (PH + 2) % 3;
+    const int Y = 2 * (n0 + i);
+    Gathered t[2];
+    if (!LEVEL0) {   // both rows' gathers in flight before the rest of the step
+      gather(Y, gkp_nxt[0], t[0]);
+      gather(imin(Y + 1, P.a.H - 1), gkp_nxt[1], t[1]);
+    }
     xpass<C>(raw);
     if (i + 3 <= nrun + 1) load_raw(i + 3, raw);
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      pin[r] = pin_nxt[r];
-      gkp[r] = gkp_nxt[r];
-    }
+    pin[0] = pin_nxt[0];
+    pin[1] = pin_nxt[1];
     if (i + 1 < nrun) load_step(i + 1, pin_nxt, gkp_nxt);
-    const int Y = 2 * (n0 + i);
-    emit<false, A, B, C>(Y, pin[0], gkp[0]);
-    if (Y + 1 < P.a.H) emit<true, A, B, C>(Y + 1, pin[1], gkp[1]);
+    emit<false, A, B, C>(Y, pin[0], t[0]);
+    if (Y + 1 < P.a.H) emit<true, A, B, C>(Y + 1, pin[1], t[1]);
   }
 
   __device__ __forceinline__ void run(int strip, int run_idx) {

@@ -9,7 +9,7 @@
 // Values are those of the per-level kernels: x pass of each row, then the y pass,
 // taps in order, clamped indices, the same point-wise expressions.
 // Bound by the barriers and shared-memory latency of one CTA: 2559x1535 RGBA, levels
-// 6 to 9 (40x24 to 5x3) and back in place of seven launches, 103.0 -> 98.6 us in all.
+// 6 to 9 (40x24 to 5x3) and back in place of six launches, 103.0 -> 98.6 us in all.
 #include <cuda_runtime.h>
 
 #include <cstring>

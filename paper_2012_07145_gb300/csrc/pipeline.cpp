@@ -1242,7 +1242,8 @@ LLLevelArgs ll_level_view_types(const hp_pipeline* p, const GroupPlan& gp) {
 }
 
 // Streaming level kernel: strips of 30 coarse columns (60 fine), tile_h coarse
-// rows per run (0: about one run per resident warp, at least 2).
+// rows per run (0: about one run per resident warp; down to one row, since a
+// coarse level's time is its rows' waits for memory one after another).
 hp_status build_ll_level_rows(const hp_pipeline* p, const Plan& plan, GroupPlan& gp, const LLLevelArgs& probe) {
   if (gp.tile_w != ll_level_rows_strip_w())
     return fail(HP_ERR_SCHEDULE, "streaming level strips are %d coarse columns wide (tile_w %d)", ll_level_rows_strip_w(),
@@ -1253,7 +1254,7 @@ hp_status build_ll_level_rows(const hp_pipeline* p, const Plan& plan, GroupPlan&
   const int strips = (cd.w + gp.tile_w - 1) / gp.tile_w;
   if (gp.tile_h == 0) {
     const long long warps = (long long)ll_level_rows_grid(probe, 1 << 30, gp.threads) * (gp.threads / 32);
-    gp.tile_h = (int)std::max(2LL, ((long long)cd.h * strips + warps - 1) / warps);
+    gp.tile_h = (int)std::max(1LL, ((long long)cd.h * strips + warps - 1) / warps);
   }
   if (gp.tile_h < 1 || gp.tile_h > 65536) return fail(HP_ERR_SCHEDULE, "streaming level needs tile_h >= 1");
   gp.grid_x = ll_level_rows_grid(probe, strips * ((cd.h + gp.tile_h - 1) / gp.tile_h), gp.threads);
@@ -1650,7 +1651,7 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
         gp.tile_h = pick(p->tile_h, g, 0);
         if (gp.tile_h == 0) {
           const long long warps = (long long)interp_rows_grid(a, 1 << 30, gp.threads) * (gp.threads / 32);
-          gp.tile_h = (int)std::max(2LL, ((long long)cd.h * strips + warps - 1) / warps);
+          gp.tile_h = (int)std::max(1LL, ((long long)cd.h * strips + warps - 1) / warps);
         }
         a.rows = gp.tile_h;
         gp.grid_x = interp_rows_grid(a, strips * ((cd.h + a.rows - 1) / a.rows), gp.threads);
