@@ -375,8 +375,11 @@ struct PlaneRun {
   }
 };
 
+// Three blocks per SM (80 registers, no spills): the rows' waits for memory overlap across
+// more warps. Against two blocks: local Laplacian 2560x1536 142.1 -> 140.1 us, interpolate
+// 2559x1535 (its first downsample) 96.7 -> 92.8, 1000x800 47.1 -> 45.8.
 template <int IDT, bool F32S>
-__global__ void __launch_bounds__(256, 2) k_ll_remap_rows(const LLRowsParams P) {
+__global__ void __launch_bounds__(256, 3) k_ll_remap_rows(const LLRowsParams P) {
   grid_dep_wait();
   __shared__ float gks[kK];
   if (threadIdx.x < kK) gks[threadIdx.x] = P.gk[threadIdx.x];
@@ -390,7 +393,7 @@ __global__ void __launch_bounds__(256, 2) k_ll_remap_rows(const LLRowsParams P) 
 
 // One level down of C f32 planes, CG channels per warp unit.
 template <int CG, bool F32S, bool PREMUL = false>
-__global__ void __launch_bounds__(256, 2) k_ll_down_rows(const LLRowsParams P) {
+__global__ void __launch_bounds__(256, 3) k_ll_down_rows(const LLRowsParams P) {
   grid_dep_wait();
   const int groups = P.a.C / CG;
   const int nw = (gridDim.x * blockDim.x) >> 5;
