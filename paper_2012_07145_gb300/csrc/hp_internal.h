@@ -354,6 +354,7 @@ int ll_level_rows_ok(const LLLevelArgs& a);
 int ll_level_rows_grid(const LLLevelArgs& a, int units, int threads);
 int launch_ll_level_rows(const LLLevelArgs& a, int rows, int threads, int grid, void* stream);
 int max_rows_strip_w();
+bool max_rows_boxed(const MaxArgs& a);
 int max_rows_grid(const MaxArgs& a, int units, int threads);
 // dynamic shared memory of the max filter kernel (the per-warp TMA rings; 0 when it loads from global memory)
 int max_rows_smem_bytes(const MaxArgs& a, int threads);

@@ -468,6 +468,9 @@ bool uses_tma(const MaxArgs& a) { return a.in.dtype == HP_F32 || a.in.dtype == H
 
 int max_rows_strip_w() { return kStripW; }
 
+// Whether the input arrives in boxes of rows, one run per warp.
+bool max_rows_boxed(const MaxArgs& a) { return uses_tma(a); }
+
 int max_rows_smem_bytes(const MaxArgs& a, int threads) {
   if (!uses_tma(a)) return 0;
   return 2 * 128 + kBarBytes + (threads / 32) * kRing * box_geom(a.in.dtype == HP_F32 ? 4 : 2).slot_bytes;

@@ -1575,7 +1575,10 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
         gp.tile_h = pick(p->tile_h, g, 0);
         if (gp.tile_h == 0) {
           const long long warps = (long long)max_rows_grid(a, 1 << 30, gp.threads) * (gp.threads / 32);
-          gp.tile_h = box_run_rows(od.h, strips * planes, warps, a.shape == 1 ? 0 : 2 * a.radius, 1 << 16);
+          // types read row by row, without boxes, keep the strided kernel's run length (8-bit
+          // 1920x1080 RGB, 3x3: 24.0 us a realize, 28.8 with runs rounded to whole boxes)
+          gp.tile_h = max_rows_boxed(a) ? box_run_rows(od.h, strips * planes, warps, a.shape == 1 ? 0 : 2 * a.radius, 1 << 16)
+                                        : default_run_rows(od.h, strips * planes, warps);
         }
         a.rows = gp.tile_h;
         gp.grid_x = max_rows_grid(a, strips * planes * ((od.h + a.rows - 1) / a.rows), gp.threads);
