@@ -267,8 +267,14 @@ int launch_interp_rows(const InterpArgs& a_in, int grid, void* stream) {
   kp.strips = (a.coarse.w + kStripW - 1) / kStripW;
   kp.units = kp.strips * ((a.coarse.h + a.rows - 1) / a.rows);
   const InterpKernel kern = pick_kernel(a);
-  int e = allow_max_dynamic_smem((const void*)kern);
-  if (e) return e;
+  // once per kernel: it is four runtime calls, and a direct launch pays them on every realize
+  static bool configured[4] = {};
+  bool& done = configured[(a.premul ? 2 : 0) + (a.final_div ? 1 : 0)];
+  if (!done) {
+    int e = allow_max_dynamic_smem((const void*)kern);
+    if (e) return e;
+    done = true;
+  }
   if (encode_tmap_3d(&kp.tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.fine.data, a.fine.w, a.fine.h, a.fine.c, a.fine.rs,
                      a.fine.ps, kBoxW, 2, 4))
     return (int)cudaErrorInvalidValue;

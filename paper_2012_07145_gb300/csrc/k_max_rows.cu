@@ -455,11 +455,19 @@ MaxKernel by_radius(int r, int shape) {
                 : r == 3 ? by_shape<IDT, 3, RND>(shape) : by_shape<IDT, 4, RND>(shape);
 }
 
-MaxKernel pick_kernel(const MaxArgs& a) {
+// The input type's index (0: f32 to f32, 1: f32 with a rounding, 2: bf16, 3: others).
+int input_kind(const MaxArgs& a) {
   const bool plain = a.st_mid == HP_F32 && a.st_out == HP_F32 && a.out.dtype == HP_F32;
-  if (a.in.dtype == HP_F32) return plain ? by_radius<HP_F32, false>(a.radius, a.shape) : by_radius<HP_F32, true>(a.radius, a.shape);
-  if (a.in.dtype == HP_BF16) return by_radius<HP_BF16, true>(a.radius, a.shape);
-  return by_radius<-1, true>(a.radius, a.shape);
+  return a.in.dtype == HP_F32 ? (plain ? 0 : 1) : a.in.dtype == HP_BF16 ? 2 : 3;
+}
+
+MaxKernel pick_kernel(const MaxArgs& a) {
+  switch (input_kind(a)) {
+    case 0: return by_radius<HP_F32, false>(a.radius, a.shape);
+    case 1: return by_radius<HP_F32, true>(a.radius, a.shape);
+    case 2: return by_radius<HP_BF16, true>(a.radius, a.shape);
+    default: return by_radius<-1, true>(a.radius, a.shape);
+  }
 }
 
 bool uses_tma(const MaxArgs& a) { return a.in.dtype == HP_F32 || a.in.dtype == HP_BF16; }
@@ -506,8 +514,14 @@ int launch_max_rows(const MaxArgs& a, int grid, void* stream) {
   const MaxKernel kern = pick_kernel(a);
   const int smem = max_rows_smem_bytes(a, a.threads);
   if (smem) {
-    int e = allow_max_dynamic_smem((const void*)kern);
-    if (e) return e;
+    // once per kernel: it is four runtime calls, and a direct launch pays them on every realize
+    static bool configured[3][4][3] = {};
+    bool& done = configured[input_kind(a)][a.radius - 1][a.shape];
+    if (!done) {
+      int e = allow_max_dynamic_smem((const void*)kern);
+      if (e) return e;
+      done = true;
+    }
     const int esize = a.in.dtype == HP_F32 ? 4 : 2;
     const CUtensorMapDataType tdt = a.in.dtype == HP_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     if (encode_tmap_3d(&kp.tmap, tdt, esize, a.in.data, a.in.w, a.in.h, a.in.c, a.in.rs, a.in.ps,
