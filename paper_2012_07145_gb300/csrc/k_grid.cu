@@ -200,9 +200,14 @@ __device__ __forceinline__ u64 lerp2(u64 a, u64 b, float f) {
 // so.  SAME: the cell size is a power of two >= 4,
 // so a thread's four pixels (rows 4 q .. 4 q + 3 of a column) lie in one cell, whose
 // corner addresses they share.  F32: the image is f32.
+// The next kernel is not let in early (grid_dep_wait, not grid_dep_sync): where
+// realizes follow one another without a graph it is the next splat, whose
+// shared memory asks for another split of the SM's memory than this kernel's
+// cache, and its waiting blocks held this grid's up (640x480: 13.7 us a realize
+// let in early, 10.0 so; 1000x700 16.5 and 12.4; replays 12.4 and 14.4 either way).
 template <bool SAME, bool F32>
 __global__ void __launch_bounds__(256) k_grid_slice_pairs(const GridArgs a) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int x = blockIdx.x * 32 + (threadIdx.x & 31);
   const int yb = blockIdx.y * 32 + (threadIdx.x >> 5) * 4;
   const int W = a.in.w, H = a.in.h;
