@@ -160,7 +160,7 @@ struct hp_pipeline {
   std::vector<int> tile_w, tile_h, threads, serial_y, impl;
   std::map<std::vector<int>, std::unique_ptr<hp::Plan>> plans;
   int* d_err = nullptr;
-  bool use_graph = false;
+  int use_graph = 0;     // HP_OPT_CUDA_GRAPH: 0, 1 or 2
   bool overlap = true;   // programmatic dependent launch between the realize's kernels
   int batch = 1;         // images per realize (a server's batched copy; see clone_pipeline)
   unsigned long long graph_replays = 0;  // realizes served by an instantiated graph
@@ -1991,15 +1991,22 @@ hp_status run_groups_impl(hp_pipeline* p, Plan& plan, const hp_buffer* inputs, c
   return HP_OK;
 }
 
-// Whether a plan is one kernel large enough to be launched directly where graph
-// replay is asked for.  Replays of one-kernel graphs follow one another with about
-// 3 us between the kernels, while a direct launch with programmatic dependent
-// launch starts as the previous kernel drains (unsharp 1023x767: 8.7 us a realize
-// against 12.3; 4-stage chain, 512x512, 11904 threads: 7.2 against 8.2).  Below 64
-// threads on each of 152 SMs the kernel is shorter than its launch takes the host,
-// and the replay is the cheaper call (max filter 300x256, 9216 threads: 7.8 us
-// direct, 6.2 replayed).
-bool launch_directly(const Plan& plan) {
+// Whether HP_OPT_CUDA_GRAPH = 1 launches a realize directly: one kernel of at
+// least 64 threads on each of 152 SMs.  In a stream of realizes, replays of
+// one-kernel graphs follow one another with 2 to 3 us between the kernels, while a
+// direct launch with programmatic dependent launch starts as the previous kernel
+// drains; a realize that is waited for alone is 1 to 2 us shorter replayed, since
+// the launch takes the host that much longer.  Both hold at every size measured,
+// 16x16 to 4096x3072 (us a realize in a stream, direct and replayed; alone,
+// direct and replayed: max filter 5x5 300x256, 7680 threads: 3.1, 6.2; 13.4, 12.2;
+// Harris 640x480, 11520 threads: 6.8, 10.2; 17.7, 16.2; unsharp 4096x3072: 51.4,
+// 55.2; 63.5, 61.5; equalization, whose cooperative launch cannot start early,
+// 640x480: 9.2 to 10.2, 10.2; 19.0, 17.0), so no size parts the two: the line takes
+// the smallest calls for ones that stand alone and the others for a stream, and
+// HP_OPT_CUDA_GRAPH = 0 or 2 has one or the other always.  Without programmatic
+// launches the stream gains 0 to 2 us only and the replay is kept.
+bool launch_directly(const hp_pipeline* p, const Plan& plan) {
+  if (!p->overlap) return false;
   const GroupPlan* only = nullptr;
   for (const GroupPlan& gp : plan.groups) {
     if (gp.folded) continue;
@@ -2239,7 +2246,7 @@ hp_status hp_realize(hp_pipeline* p, const hp_buffer* inputs, int n_inputs, cons
   if ((s = check_buffer(*output, os.storage, os.channels * p->batch, plan->dom[p->output], "output", 0))) return s;
   if (!p->d_err && (s = alloc_error_word(p, stream))) return s;
   if ((s = ensure_scratch(p, *plan, (cudaStream_t)stream))) return s;
-  if (!p->use_graph || launch_directly(*plan)) return run_groups(p, *plan, inputs, output, stream);
+  if (!p->use_graph || (p->use_graph == 1 && launch_directly(p, *plan))) return run_groups(p, *plan, inputs, output, stream);
   return run_graph(p, *plan, inputs, n_inputs, output, stream);
 }
 
@@ -2572,16 +2579,18 @@ hp_status hp_check_device_error(hp_pipeline* p, int* code) {
 hp_status hp_set_option(hp_pipeline* p, int option, long long value) {
   if (!p) return fail(HP_ERR_INVALID_ARG, "null pipeline");
   switch (option) {
-    case HP_OPT_CUDA_GRAPH:
-      if (p->use_graph != (value != 0)) {
+    case HP_OPT_CUDA_GRAPH: {
+      const int mode = value == 2 ? 2 : value != 0;
+      if (p->use_graph != mode) {
         for (auto& kv : p->plans) {
           for (auto& g : kv.second->graphs) cudaGraphExecDestroy(g.exec);
           kv.second->graphs.clear();
           kv.second->seen.clear();
         }
       }
-      p->use_graph = value != 0;
+      p->use_graph = mode;
       return HP_OK;
+    }
     case HP_OPT_OVERLAP:
       if (p->overlap != (value != 0)) {  // captured graphs hold the old launch attributes
         for (auto& kv : p->plans) {

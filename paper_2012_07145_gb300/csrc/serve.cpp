@@ -155,7 +155,7 @@ hp_pipeline* slot_clone(Slot& sl, hp_pipeline* p, int batch) {
   auto it = sl.clones.find(key);
   if (it != sl.clones.end()) return it->second;
   hp_pipeline* c = hp::clone_pipeline(p, batch);
-  if (c) hp_set_option(c, HP_OPT_CUDA_GRAPH, 1);  // a slot's realize of a shape replays as a graph
+  if (c) hp_set_option(c, HP_OPT_CUDA_GRAPH, 2);  // a slot's realize of a shape replays as a graph, one kernel or more
   sl.clones[key] = c;
   return c;
 }

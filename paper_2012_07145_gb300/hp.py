@@ -275,8 +275,10 @@ class Pipeline:
     def set_option(self, option: int, value: int):
         check(lib().hp_set_option(self.h, option, value))
 
-    def use_cuda_graph(self, on: bool = True):
-        self.set_option(HP_OPT_CUDA_GRAPH, 1 if on else 0)
+    def use_cuda_graph(self, on: bool = True, always: bool = False):
+        """Realizes as graph replays; all but the smallest realizes of one kernel are launched
+        directly unless `always` (HP_OPT_CUDA_GRAPH)."""
+        self.set_option(HP_OPT_CUDA_GRAPH, (2 if always else 1) if on else 0)
 
     def overlap_launches(self, on: bool = True):
         """Programmatic dependent launch between the realize's kernels (the default)."""
