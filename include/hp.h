@@ -137,7 +137,17 @@ typedef struct {
  * computes every member over the tile its output needs, keeping members in
  * shared memory or registers; only the group's output stage (the one stage read
  * outside the group, or the pipeline output) is written to memory.  Singleton
- * groups everywhere is the stage-per-kernel schedule ("compute root", Sec. 2). */
+ * groups everywhere is the stage-per-kernel schedule ("compute root", Sec. 2).
+ *
+ * Lowering for given sizes folds two kinds of groups into others; the values do
+ * not change.  A premultiply that only streaming interpolate levels and streaming
+ * 4-channel downsamples read is recomputed in them.  The streaming downsamples and
+ * level steps of a pyramid's coarse end (three or more levels of at most 1024
+ * pixels that nothing else reads) run as one launch, reported as its finest step's.
+ * The tile, threads and rows that the schedule gives a folded group do not apply;
+ * a group that another kernel takes (HP_IMPL_GENERIC, or a downsample or
+ * local-Laplacian level of a tile_w other than 30) is not folded.
+ * hp_group_info_get reports a folded group with a grid of 0. */
 enum {
   HP_IMPL_AUTO = 0,    /* the kernel the group's shape selects */
   HP_IMPL_GENERIC = 1, /* the generic interpreter */
@@ -193,9 +203,12 @@ typedef struct {
   long long plane_stride_bytes;/* multiple of 16 */
 } hp_buffer;
 
-/* Per-group facts after lowering, for tests and the tuner. */
+/* Per-group facts after lowering, for tests and the tuner.  A group folded into
+ * others (see hp_schedule) has no launch: its grid, threads and smem_bytes are 0.
+ * A level step that launches a pyramid's coarse end has the facts of that launch:
+ * one CTA, smem_bytes of all its levels, tile_w x tile_h its finest level. */
 typedef struct {
-  int kernel;                  /* hp_kernel_id below */
+  int kernel;                  /* hp_kernel_id below: the kernel the group's shape and schedule select */
   int output_stage;
   int n_members;               /* stages computed in the group (inlined ones included) */
   int tile_w, tile_h, threads;

@@ -364,6 +364,7 @@ int interp_rows_grid(const InterpArgs& a, int units, int threads);
 // dynamic shared memory of the interpolate level kernel (the per-warp TMA rings of the fine level)
 int interp_rows_smem_bytes(int threads);
 int launch_interp_rows(const InterpArgs& a, int grid, void* stream);
+int pyr_tail_threads();
 int pyr_tail_smem_bytes(const PyrTailArgs& a);
 int launch_pyr_tail(const PyrTailArgs& a, void* stream);
 int pw_rows_op_ok(int op);

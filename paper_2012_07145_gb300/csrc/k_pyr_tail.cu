@@ -142,6 +142,8 @@ long long layout(const PyrTailArgs& a, int* off, int* roff) {
 
 }  // namespace
 
+int pyr_tail_threads() { return kThreads; }
+
 // Shared memory of a tail, or 0 where it does not fit one CTA.
 int pyr_tail_smem_bytes(const PyrTailArgs& a) {
   int off[kTailLevels], roff[kTailLevels];

@@ -1692,6 +1692,18 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
   plan_grid_pairs(p, plan);
   if ((s = plan_premul_fold(p, plan))) return s;
   plan_pyr_tail(p, plan);
+  // the launches as they are: none for a folded group, one CTA for a tail
+  for (GroupPlan& gp : plan.groups) {
+    if (gp.folded) {
+      gp.grid_x = gp.grid_y = gp.grid_z = gp.threads = gp.smem = 0;
+    } else if (gp.tail) {
+      gp.tile_w = gp.tail_args.w[0];
+      gp.tile_h = gp.tail_args.h[0];
+      gp.grid_x = gp.grid_y = gp.grid_z = 1;
+      gp.threads = pyr_tail_threads();
+      gp.smem = pyr_tail_smem_bytes(gp.tail_args);
+    }
+  }
   return HP_OK;
 }
 
