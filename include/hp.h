@@ -147,7 +147,7 @@ typedef struct {
  * The tile, threads and rows that the schedule gives a folded group do not apply;
  * a group that another kernel takes (HP_IMPL_GENERIC, or a downsample or
  * local-Laplacian level of a tile_w other than 30) is not folded.
- * hp_group_info_get reports a folded group with a grid of 0. */
+ * hp_group_info_get reports a folded group with grid_z = 0. */
 enum {
   HP_IMPL_AUTO = 0,    /* the kernel the group's shape selects */
   HP_IMPL_GENERIC = 1, /* the generic interpreter */
@@ -204,7 +204,8 @@ typedef struct {
 } hp_buffer;
 
 /* Per-group facts after lowering, for tests and the tuner.  A group folded into
- * others (see hp_schedule) has no launch: its grid, threads and smem_bytes are 0.
+ * others (see hp_schedule) has no launch: its grid_z is 0, and the rest are the
+ * facts its own launch would have had.
  * A level step that launches a pyramid's coarse end has the facts of that launch:
  * one CTA, smem_bytes of all its levels, tile_w x tile_h its finest level. */
 typedef struct {

@@ -1695,7 +1695,7 @@ hp_status lower(hp_pipeline* p, const std::vector<Dom>& in_dom, Plan& plan) {
   // the launches as they are: none for a folded group, one CTA for a tail
   for (GroupPlan& gp : plan.groups) {
     if (gp.folded) {
-      gp.grid_x = gp.grid_y = gp.grid_z = gp.threads = gp.smem = 0;
+      gp.grid_z = 0;
     } else if (gp.tail) {
       gp.tile_w = gp.tail_args.w[0];
       gp.tile_h = gp.tail_args.h[0];

@@ -1,5 +1,5 @@
 """hp_group_info_get against what a realize launches: groups folded into others
-have no launch, a pyramid's coarse end is one CTA."""
+have no launch (grid_z = 0), a pyramid's coarse end is one CTA."""
 
 import pytest
 
@@ -17,15 +17,7 @@ def facts(p, w, h):
 
 
 def launched(infos):
-    return [i for i in infos if i.grid_x * i.grid_y * i.grid_z > 0]
-
-
-def check_facts(infos):
-    for i in infos:
-        if i.grid_x * i.grid_y * i.grid_z == 0:
-            assert (i.grid_x, i.grid_y, i.grid_z, i.threads, i.smem_bytes) == (0, 0, 0, 0, 0)
-        else:
-            assert i.threads > 0
+    return [i for i in infos if i.grid_z > 0]
 
 
 def tails(infos):
@@ -58,7 +50,7 @@ def test_facts_of_folded_groups(app, w, h, levels, finest):
     inside = [s for s in sizes[1:] if s[0] * s[1] <= 1024]
     p = build(app, levels)
     infos = facts(p, w, h)
-    check_facts(infos)
+    assert all(i.grid_x > 0 and i.grid_y > 0 and i.grid_z >= 0 and i.threads >= 32 for i in infos)
     premul = 1 if app == "interpolate" else 0
     saved = 2 * (len(inside) - 1) - 1 if len(inside) >= 3 else 0
     assert len(launched(infos)) == p.group_count() - premul - saved
