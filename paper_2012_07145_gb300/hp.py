@@ -249,8 +249,11 @@ class Pipeline:
     def realize(self, inputs, output, stream=None):
         """inputs: list of Buffer (device); output: Buffer (device); stream: cudaStream_t as int or None."""
         n = len(inputs)
-        arr = ctypes.byref(inputs[0]) if n == 1 else (Buffer * n)(*inputs)   # one buffer is its own array
-        st = _lib.hp_realize(self.h, arr, n, ctypes.byref(output), stream)
+        if n == 1 and type(inputs) is list and type(inputs[0]) is Buffer:
+            arr = ctypes.byref(inputs[0])   # one buffer is its own array (0.3 us, 0.95 as a new one)
+        else:
+            arr = (Buffer * n)(*inputs)
+        st = _lib.hp_realize(self.h, arr, n, ctypes.byref(output), ctypes.c_void_p(stream or 0))
         if st != HP_OK:
             check(st)
 
