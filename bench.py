@@ -759,7 +759,7 @@ def run_ours(args, cfg_name):
         "config": {"workload": cfg["workload"],
                    "schedule": schedule_of(cfg_name, cfg),
                    "l2": "flushed between timed steps (256 MiB written, then read back: clean lines)", "parallelism": f"replicas x{world}",
-                   "launch": "CUDA graph replay"},
+                   "launch": "CUDA graph replay" if r["launches"] > args.steps else "direct launch (one kernel)"},
         "plain": {"value": round(npx / (r["plain_ms"] * 1e-3) / 1e6, 2), "unit": "MPix/s",
                   "ms_per_step": round(r["plain_ms"], 5),
                   "launches_per_step": r["plain_launches"] / r["plain_steps"],

@@ -241,12 +241,15 @@ enum {
                                   (gray, K = 8 remaps, downsample), streaming: one warp per strip
                                   of 30 coarse columns, everything in registers */
   HP_KERNEL_LL_DOWN_ROWS = 16,  /* one pyramid level down of a stack of f32 planes, streaming: one
-                                  warp per strip of 30 coarse columns and 3 (or 1) planes */
+                                  warp per strip of 30 coarse columns and 3 (or 1) planes, or the 4 of an
+                                   RGBA image that it premultiplies */
   HP_KERNEL_LL_LEVEL_ROWS = 17, /* local-Laplacian level (K = 8, f32 stages), streaming: one warp per
                                   strip of 30 coarse (60 fine) columns, upsample window in shared memory */
   HP_KERNEL_MAX_ROWS = 18,      /* max filter (one square window-maximum stage of radius 1..4, or a
                                   horizontal and a vertical one), streaming: one warp per strip of 120
-                                  columns of one plane, a ring of row maxima in registers */
+                                  columns of one plane; f32 and bf16 rows through a per-warp TMA
+                                  ring, prefix and suffix maxima of blocks of 4 rows; other types
+                                  a ring of row maxima in registers */
   HP_KERNEL_INTERP_ROWS = 19,   /* interpolate level (upsample, composite, optional division by
                                   coverage; f32 RGBA), streaming: one warp per strip of 30 coarse
                                   columns, upsample window in registers */
@@ -255,7 +258,7 @@ enum {
                                   thread, 128-bit loads and stores */
   HP_KERNEL_GRID_SPLAT = 21,    /* bilateral grid splat: one thread per cell (four, two pixel rows
                                   each, for 8 x 8 cells), accumulators in shared memory */
-  HP_KERNEL_GRID_SLICE = 22,    /* bilateral grid slice: four pixels of a row per thread, trilinear */
+  HP_KERNEL_GRID_SLICE = 22,    /* bilateral grid slice: four pixels per thread, trilinear */
   HP_KERNEL_GRID_BLUR = 23,     /* bilateral grid blur (range levels, x, y; binomial/16), streaming:
                                   one warp per 28 grid columns x 4 range levels, y taps in order */
   HP_KERNEL_STENCIL_LINES = 24  /* fused chain of 5x5 stencils, line-buffered: every stage on threads of
@@ -371,7 +374,7 @@ hp_status hp_kernel_attrs_get(hp_pipeline* p, int* n_kernels, int* max_registers
  * `max_batch` queued requests for the same pipeline, image size and buffer
  * kind, with at most 32 MB of inputs and outputs in all, are served by one
  * realize: their images are stacked as planes, so each
- * kernel launches once, as one persistent grid, for the batch, and every
+ * kernel launches once, as one grid, for the batch, and every
  * result equals the request's solo result.  Batching covers pipelines whose
  * stages act on each channel separately (stencils, resampling, per-channel
  * point-wise ops) and the fused Harris and histogram-equalization kernels.

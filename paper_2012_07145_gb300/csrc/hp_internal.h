@@ -261,8 +261,9 @@ struct LLLevelArgs {
 // level 0 of the tail is read, its result (I or R) written.
 constexpr int kTailLevels = 16;
 constexpr int kTailPixels = 1024;   // of the tail's finest level: larger ones keep one CTA busy for longer than their
-                                    // launches take (interpolate 2559x1535, 10 levels: 103.0 us without a tail, 98.6 at
-                                    // 1024, 104.4 at 4096; 400x300, 8 levels: 35.5, 30.7, 33.1)
+                                    // launches take (us at 512, 1024, 2048 and 4096; interpolate, 10 levels, 1000x700:
+                                    // 41.6, 40.3, 40.3, 43.7; 400x300: 27.7, 27.7, 29.8, 29.7; local Laplacian, 8
+                                    // levels, 1000x700: 59.5, 56.9, 56.9, 63.0; 400x300: 36.8, 36.8, 41.9, 41.8)
 struct PyrTailArgs {
   ImgView src, out;
   int levels, channels;    // channels of a level's stack

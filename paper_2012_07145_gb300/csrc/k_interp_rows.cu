@@ -13,9 +13,9 @@
 // Lanes 0 and 31 only feed their neighbours.  The two fine rows of D_l a
 // coarse step composites arrive as one TMA box (68 fine columns from a 16-byte
 // aligned start, 2 rows, the 4 planes) through a ring of 3 shared-memory slots
-// private to the warp, issued in the order the warp will read them (across its
-// runs), so the fine loads are in flight well ahead of their use without
-// holding registers.  The operations are those of the
+// private to the warp (a warp runs one run): three are issued with the run, each
+// next one once its slot is read, so the fine loads are in flight well ahead of
+// their use without holding registers.  The operations are those of the
 // per-pixel expressions (x pass over each coarse row, then the y pass, in tap
 // order; op_over, op_unpremul), so results are bit-identical to the generic
 // kernel.  All stages are stored as f32 (the host checks).

@@ -14,8 +14,8 @@
 // channel separately (stencils, per-channel point-wise ops, resampling) simply
 // see more channels; the fused Harris and histogram-equalization kernels take
 // the batch as an image index (each image keeps its own planes, and for the
-// histogram its own counters and table).  The kernels of a batch are
-// persistent: one grid sized to the GPU walks every image's work units.
+// histogram its own counters and table): one grid has every image's work units,
+// a run of rows per warp, or for the histogram a range of each image per CTA.
 //
 // Residency: each slot keeps, per (pipeline, batch size, image size), a
 // staging region in the HBM arena reserved at creation, and keeps it after

@@ -244,8 +244,8 @@ def apply_entry(p, ids, pipeline, entry):
 
 # ------------------------------------------------------------------ timing --
 def time_candidate(p, bi, bo, stream, flush, reps=15, probe=False):
-    """Median ms of `reps` graph replays (L2 flushed before each: written and
-    read back); with probe, also the (kernels, max registers, max local bytes)
+    """Median ms of `reps` realizes, replayed or launched as HP_OPT_CUDA_GRAPH = 1
+    has it (L2 flushed before each: written and read back); with probe, also the (kernels, max registers, max local bytes)
     of the launched kernels."""
     import torch
     s = stream.cuda_stream
@@ -273,7 +273,7 @@ def time_candidate(p, bi, bo, stream, flush, reps=15, probe=False):
 
 
 def burst_ms(wl, p, ids, c, bi, bo, stream, n=200):
-    """Mean ms of back-to-back graph replays of candidate c (best of 3 bursts)."""
+    """Mean ms of back-to-back realizes of candidate c (best of 3 bursts)."""
     import torch
     wl["apply"](p, ids, c)
     best = float("inf")
@@ -346,7 +346,7 @@ def tune(pipeline, w, h, dtype, quick=False, log=print):
     results.sort(key=lambda r: r[0])
     best = results[0]
     # event times come in steps of about 2 us: candidates on the best's step are
-    # told apart by bursts of replays, the first listed within 2% taken
+    # told apart by bursts of realizes, the first listed within 2% taken
     near = sorted((r for r in results if r[0] <= best[0] + 0.0006), key=lambda r: order[id(r[1])])[:40]
     if best[0] < 0.05 and len(near) > 1:
         bursts = [burst_ms(wl, p, ids, r[1], bi, hp.buffer_from_tensor(y, odt), stream) for r in near]
