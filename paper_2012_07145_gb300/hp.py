@@ -253,7 +253,9 @@ class Pipeline:
             arr = ctypes.byref(inputs[0])   # one buffer is its own array (0.3 us, 0.95 as a new one)
         else:
             arr = (Buffer * n)(*inputs)
-        st = _lib.hp_realize(self.h, arr, n, ctypes.byref(output), ctypes.c_void_p(stream or 0))
+        if type(stream) is not int:
+            stream = ctypes.c_void_p(stream or 0)   # None, or refused
+        st = _lib.hp_realize(self.h, arr, n, ctypes.byref(output), stream)
         if st != HP_OK:
             check(st)
 
