@@ -12,6 +12,12 @@
 // expressions and per-stage rounding are those of stage_math.cuh, so the result
 // is bit-identical to every other schedule of the pipeline.
 //
+// A warp runs one run, with a ring of that run, and every lane tests a box's
+// barrier itself.  Bound by issue (115 to 120 registers, two CTAs of 256 per SM):
+// 2560x1536 RGB f32 takes 17.5 us in a stream of realizes (0.53 of the measured
+// copy rate); as replays, with a ring across a warp's runs that one lane waited on,
+// 640x480 took 10.3 us and 4096x3072 54, with a run's own 8.2 and 44.
+//
 // Boundary conditions (each stencil clamps on its own producer, Sec. 3): an x
 // pass at the image's first or last column takes the edge column itself as the
 // missing neighbour (a select on the shuffled value); rows outside take the

@@ -19,10 +19,10 @@
 //     column for any radius), not as 2r + 1 rows.
 // A warp runs one unit and every lane tests the box's barrier itself, so the
 // ring needs no bookkeeping across units.  Bound by the loads' latency, then by
-// memory: 2560x1536 RGB f32 9x9 takes 20.6 us (94 MB: 0.68 of the measured copy
-// rate), against 39.3 with 2r + 1 rows of maxima in registers, a row loop
-// unrolled as often, and a ring across units that one lane waited on; with the
-// blocks but that ring it was 31.8.
+// memory: 2560x1536 RGB f32 9x9 takes 17.5 us in a stream of realizes (94 MB: 0.80
+// of the measured copy rate).  As graph replays it is 20.6, against 39.3 with
+// 2r + 1 rows of maxima in registers, a row loop unrolled as often, and a ring
+// across units that one lane waited on; with the blocks but that ring it was 31.8.
 //
 // Other input types: one warp per strip of 120 columns, rows loaded from global
 // memory, the next row's loads in flight while a row is processed; the
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(256, max_rows_min_blocks<RX, RY>()) k_max_rows
 }
 
 // Two CTAs of 8 warps per SM: 96 KB of boxes in flight are enough, and more CTAs
-// would spill (2560x1536 RGB f32 9x9: 20.6 us at two, 22.4 at three, 24.7 at four).
+// would spill (2560x1536 RGB f32 9x9, replayed: 20.6 us at two, 22.4 at three, 24.7 at four).
 template <int IDT, int RX, int RY, bool RND>
 __global__ void __launch_bounds__(256, 2) k_max_rows_tma(const __grid_constant__ MaxParams P) {
   grid_dep_wait();

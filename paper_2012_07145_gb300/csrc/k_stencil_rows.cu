@@ -13,6 +13,9 @@
 // blocks, alternating, so nothing is moved), and the unsharp combine keeps the
 // two input rows it is behind.  The stencil and combine expressions are those of
 // stage_math.cuh, so the result is bit-identical to every other schedule.
+// Bound by memory: unsharp 4096x3072 RGB f32 takes 47.2 us in a stream of realizes
+// (302 MB: 0.94 of the measured copy rate), 50.4 replayed; with the ring across
+// units, one row at a time and a queue of row registers, 68.7 replayed.
 //
 // Boundary condition (clamp to edge on the stencil's input): in strips that
 // touch the left or right image edge the two columns outside it are written into
