@@ -250,12 +250,14 @@ class Pipeline:
         """inputs: list of Buffer (device); output: Buffer (device); stream: cudaStream_t as int or None."""
         n = len(inputs)
         if n == 1 and type(inputs) is list and type(inputs[0]) is Buffer:
-            arr = ctypes.byref(inputs[0])   # one buffer is its own array (0.3 us, 0.95 as a new one)
+            arr = inputs[0]                 # passed by reference: one buffer is its own array
         else:
             arr = (Buffer * n)(*inputs)
+        if type(output) is not Buffer:
+            output = ctypes.byref(output)
         if type(stream) is not int:
             stream = ctypes.c_void_p(stream or 0)   # None, or refused
-        st = _lib.hp_realize(self.h, arr, n, ctypes.byref(output), stream)
+        st = _lib.hp_realize(self.h, arr, n, output, stream)
         if st != HP_OK:
             check(st)
 
